@@ -50,7 +50,7 @@ Layout make_layout(const mira_config& c) {
     L.sum_pos = o;   o = align256(o + (T >= (size_t)kTensorPathMinTokens ? P * 4 : 0));
     L.h16 = o;       o = align256(o + P * R * 2);
     L.h16lo = o;     o = align256(o + P * R * 2);
-    L.ypart = o;     o = align256(o + std::max(S * P * C * 4, R * 4));   // at least one expert's abs-max scratch for the quantizer
+    L.ypart = o;     o = align256(o + S * P * C * 4);
     L.pred = o;      o = align256(o + T * E * 4);
     L.mix = o;       o = align256(o + 8 * (C + E) * 4);
     L.tickets = o;   o = align256(o + (T / 8 + 1) * 4);
@@ -214,7 +214,6 @@ mira_status mira_create(const mira_config* cfg, void* dev_workspace, size_t work
     if ((s = set_ffn_attributes()) != MIRA_OK) return s;
     if ((s = set_tc_attributes()) != MIRA_OK) return s;
     if ((s = set_mixture_attributes()) != MIRA_OK) return s;
-    if ((s = set_quantize_attributes()) != MIRA_OK) return s;
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.status, 0, 32 * sizeof(int32_t)));
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.tickets, 0, ((size_t)cfg->max_tokens / 8 + 1) * 4));
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.sched, 0, sizeof(Sched)));   // the up/gate kernel's rehearsal pass reads it before the first schedule is written

@@ -195,7 +195,6 @@ mira_status launch_mixture(mira_ctx*, const void* hidden, int T, const float* lo
                            int32_t* out_ids, int k_pred, cudaStream_t);
 mira_status set_mixture_attributes();
 mira_status set_ffn_attributes();
-mira_status set_quantize_attributes();
 
 // api.cu: the pieces of a layer step for the stack runtime, which starts the resident experts before the host has
 // read the routing counts. route_and_schedule = S1-S3 plus the schedule over every routed expert that slot_map
