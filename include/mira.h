@@ -130,7 +130,8 @@ mira_status mira_stage_expert(mira_ctx* ctx, const void* pinned_host_blob, void*
 
 /* Section IV-E, linear head on the hidden state: scores the experts of layer `layer + 2`.
  *   token score[t][e] = sum_c hidden[t][c] * pred_w[e][c] + pred_b[e]      (fp32 accumulation)
- *   out_expert_scores[e] = mean over t (fp32; 32 interleaved partial sums over the tokens, added pairwise, divided by T)
+ *   out_expert_scores[e] = mean over t (fp32; taken over the token scores if they are asked for, else over the tokens first:
+ *                          the same number up to fp32 rounding, without a score per token)
  *   out_topk_ids = the k_pred best pooled scores, ties to the lower id.
  * hidden [T][C] bf16, pred_w [E][C] bf16, pred_b [E] fp32 or NULL, out_token_scores [T][E] or NULL,
  * out_topk_ids [k_pred] or NULL (then k_pred is ignored). Heads exist for every layer except the
@@ -147,8 +148,8 @@ mira_status mira_predict(mira_ctx* ctx, int32_t layer, const void* hidden, int32
  * serving loop whose memory plan is frozen, a plug-in that is handed tensors but no allocator, a
  * process whose device memory is fully pre-partitioned. They cannot create a mira_ctx, because a
  * context needs a caller-provided device workspace. This variant of mira_predict needs neither: it
- * takes plain input and output pointers and keeps its only scratch (the per-token scores, T * E
- * floats) in a fixed array that is part of the library image, MIRA_NOALLOC_MAX_SCORES floats
+ * takes plain input and output pointers and keeps its only scratch (sums over groups of
+ * tokens) in a fixed array that is part of the library image, MIRA_NOALLOC_MAX_SCORES floats
  * (256 KB) on every GPU that loads the library, held until the process exits.
  *
  *   out_expert_scores[e] = mean over t of (sum_c hidden[t][c] * pred_w[e][c] + pred_b[e]);
@@ -158,7 +159,7 @@ mira_status mira_predict(mira_ctx* ctx, int32_t layer, const void* hidden, int32
  * fp32 device or NULL, outputs device. Limits: T * n_experts <= MIRA_NOALLOC_MAX_SCORES (else
  * MIRA_ERR_WORKSPACE), hidden_size % 8 == 0 and <= 16384, n_experts <= 256, k_pred <= 16.
  * The call allocates and frees nothing, on the host allocator of CUDA or on the device. The first call
- * on each device resolves the device address of the scratch array and raises a kernel attribute; make
+ * on each device resolves the device address of the scratch array; make
  * that first call outside any stream capture. All calls on one GPU share the scratch array, which
  * keeps the previous call's contents (every entry a call reads it has written first, so nothing needs
  * clearing): two calls whose kernels can overlap on the GPU (different streams) race on it -- keep
@@ -225,7 +226,7 @@ mira_status mira_profile_read(mira_ctx* ctx, float* total_ms, int64_t* launches)
 /* Section IV-E, MixtureHead: the predictor as a mixture of an activation branch and a history branch with a
  * contextual gate. The paper names the parts and the features but no sizes or non-linearities; this is the smallest
  * instance with every named part, all branches linear (E2 = experts of the predicted layer, here E2 = E):
- *   hbar = mean_t hidden[t][:]      lbar = mean_t router_logits[t][:]      (means summed in token order)
+ *   hbar = mean_t hidden[t][:]      lbar = mean_t router_logits[t][:]      (fp32)
  *   hist[e] = count[e] / sum_e count[e] over the routed experts      top[e] = 1 for the k_top largest counts
  *                                                                    (ties to the lower id), else 0
  *   act = wa_h hbar + wa_l lbar + b_a          (ActHead)        his = wh_c hist + wh_t top + b_h      (HistHead)

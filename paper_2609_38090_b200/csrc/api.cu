@@ -51,8 +51,9 @@ Layout make_layout(const mira_config& c) {
     L.h16 = o;       o = align256(o + P * R * 2);
     L.h16lo = o;     o = align256(o + P * R * 2);
     L.ypart = o;     o = align256(o + S * P * C * 4);
-    L.pred = o;      o = align256(o + T * E * 4);
-    L.mix = o;       o = align256(o + 8 * (C + E) * 4);
+    const size_t head_floats = std::min<size_t>(64 * (C + E), std::max<size_t>(C + E, MIRA_NOALLOC_MAX_SCORES));      // head_chunks of any T
+    L.pred = o;      o = align256(o + head_floats * 4);
+    L.mix = o;       o = align256(o + head_floats * 4);
     L.tickets = o;   o = align256(o + (T / 8 + 1) * 4);
     L.total = o;
     return L;
@@ -213,7 +214,6 @@ mira_status mira_create(const mira_config* cfg, void* dev_workspace, size_t work
     if ((s = set_route_attributes()) != MIRA_OK) return s;
     if ((s = set_ffn_attributes()) != MIRA_OK) return s;
     if ((s = set_tc_attributes()) != MIRA_OK) return s;
-    if ((s = set_mixture_attributes()) != MIRA_OK) return s;
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.status, 0, 32 * sizeof(int32_t)));
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.tickets, 0, ((size_t)cfg->max_tokens / 8 + 1) * 4));
     MIRA_CUDA_OK(cudaMemset(static_cast<char*>(dev_workspace) + L.sched, 0, sizeof(Sched)));   // the up/gate kernel's rehearsal pass reads it before the first schedule is written
@@ -300,10 +300,18 @@ mira_status mira_predict(mira_ctx* ctx, int32_t layer, const void* hidden, int32
     if (misaligned(hidden) || misaligned(pred_w)) return MIRA_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int E = ctx->cfg.n_experts;
-    float* ts = out_token_scores ? out_token_scores : ws_ptr<float>(ctx, ctx->lay.pred);
-    mira_status s = launch_scores(ctx, hidden, T, pred_w, pred_b, E, ts, nullptr, nullptr, nullptr, st);
+    if (!out_token_scores) {
+        int n = 0;
+        ProfScope ps(ctx, MIRA_K_SCORES, st);
+        const mira_status s = launch_linear_head(hidden, T, ctx->cfg.hidden, pred_w, pred_b, E, out_expert_scores, out_topk_ids,
+                                                 out_topk_ids ? k_pred : 0, ws_ptr<float>(ctx, ctx->lay.pred), ctx->notify_ids,
+                                                 ctx->notify_ids_flag, ctx->notify_seq, st, &n);
+        ctx->launches += n;
+        return s;
+    }
+    mira_status s = launch_scores(ctx, hidden, T, pred_w, pred_b, E, out_token_scores, nullptr, nullptr, nullptr, st);
     if (s != MIRA_OK) return s;
-    return launch_pool(ctx, ts, T, E, out_expert_scores, out_topk_ids, out_topk_ids ? k_pred : 0, st);
+    return launch_pool(ctx, out_token_scores, T, E, out_expert_scores, out_topk_ids, out_topk_ids ? k_pred : 0, st);
 }
 
 mira_status mira_predict_mixture(mira_ctx* ctx, int32_t layer, const void* hidden, int32_t T, const float* router_logits,

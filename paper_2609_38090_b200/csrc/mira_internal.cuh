@@ -88,8 +88,8 @@ struct Layout {
     size_t sum_pos;     // float [Pmax]    per position: sum of the token's fp16 activations (tensor-core path)
     size_t h16;         // half  [Pmax][R]
     size_t ypart;       // float [S][Pmax][C] split partial sums of the down projection
-    size_t pred;        // float [Tmax][E] per-token predictor scores when the caller passes none
-    size_t mix;         // float [8][C + E] partial column sums of the MixtureHead's mean features
+    size_t pred;        // float [head_chunks][C + E] token sums of the linear head's batches ...
+    size_t mix;         // ... and of the MixtureHead's
     size_t tickets;     // uint32 [Tmax / 8 + 1] arrival counters of the 2-D score kernel, one per token group (zero at rest)
     size_t total;
 };
@@ -137,7 +137,7 @@ struct mira_ctx {
     int32_t* notify_count = nullptr;
     uint32_t* notify_flag = nullptr;
     uint32_t notify_seq = 0;
-    int32_t* notify_ids = nullptr;      // likewise for the pooling kernel's top-k ids (mira_predict)
+    int32_t* notify_ids = nullptr;      // likewise for the linear head's top-k ids (mira_predict)
     uint32_t* notify_ids_flag = nullptr;
 };
 
@@ -189,11 +189,14 @@ inline int tc_min_tokens_down(const mira_config& c) { return c.n_experts + c.n_s
 // kernel (0: every expert; INT_MAX: none). The same rule for every wave of a routed batch.
 void step_tc_min(const mira_ctx* ctx, int T, int k, int out_min[2]);
 mira_status set_route_attributes();
-// mixture_head.cu
+// predictor.cu
+int head_chunks(int T, int C, int E);
+mira_status launch_linear_head(const void* hidden, int T, int C, const void* w, const float* b, int E, float* out_scores,
+                               int32_t* out_ids, int k_pred, float* part, int32_t* host_ids, uint32_t* host_flag,
+                               uint32_t host_seq, cudaStream_t, int* launches);
 mira_status launch_mixture(mira_ctx*, const void* hidden, int T, const float* logits, const int32_t* count, int k_top,
                            const mira_mixture_head& head, float* out_scores, float* out_probs, float* out_alpha,
                            int32_t* out_ids, int k_pred, cudaStream_t);
-mira_status set_mixture_attributes();
 mira_status set_ffn_attributes();
 
 // api.cu: the pieces of a layer step for the stack runtime, which starts the resident experts before the host has
@@ -242,6 +245,38 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+// Top-k by a warp.
+// The selection runs on 32-bit keys that order like the logits (sign-magnitude floats mapped to unsigned; -0 counts as
+// +0, a NaN ranks below every number), with two hardware warp reductions per selected expert: the largest key, then
+// the lowest index that holds it. Keys: 0 = no candidate (beyond E, or already selected), 1 = NaN, else the logit.
+// SLOTS = values per lane that can be occupied (2 covers 64 experts): this code runs once per token on the critical
+// path of a decode step, where every instruction is fetched cold, so the short form matters.
+__device__ __forceinline__ unsigned topk_key(float v) {
+    if (!(v == v)) return 1u;
+    const unsigned b = __float_as_uint(v + 0.f);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float topk_value(unsigned key) {
+    if (key <= 1u) return key ? __uint_as_float(0x7fc00000u) : -INFINITY;
+    return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+}
+// One selection step: returns the winner's index and key to every lane and retires it. With nothing left the result is
+// index 0 with key 0.
+template <int SLOTS>
+__device__ __forceinline__ void topk_step(unsigned (&key)[SLOTS], int lane, int& win_idx, unsigned& win_key) {
+    unsigned bk = 0u;
+#pragma unroll
+    for (int i = 0; i < SLOTS; ++i) bk = max(bk, key[i]);
+    win_key = __reduce_max_sync(0xffffffffu, bk);
+    unsigned cand = 0xffffffffu;
+#pragma unroll
+    for (int i = SLOTS - 1; i >= 0; --i) if (key[i] == win_key) cand = (unsigned)(lane + 32 * i);
+    const unsigned w = __reduce_min_sync(0xffffffffu, win_key ? cand : 0xffffffffu);
+    win_idx = (w == 0xffffffffu) ? 0 : (int)w;
+#pragma unroll
+    for (int i = 0; i < SLOTS; ++i) if (win_key && lane + 32 * i == win_idx) key[i] = 0u;
+}
 #endif
 
 #define MIRA_CUDA_OK(expr) do { cudaError_t e__ = (expr); if (e__ != cudaSuccess) return MIRA_ERR_CUDA; } while (0)

@@ -32,8 +32,6 @@ __device__ __forceinline__ float dot8(const uint4& a, const uint4& b, float acc)
     return acc;
 }
 
-// Warp top-k over up to 256 values held 8 per lane (value j of lane l is element l + 32 j).
-// Order: value descending, index ascending. Lane 0 returns through out_idx / out_val (k <= 16).
 // Warps walk the router rows in rounds (row w, w + nwarps, ...). The rows of the later rounds are requested
 // into L2 up front, so that after a step that streamed the experts through L2 only the first round pays DRAM
 // latency.
@@ -43,37 +41,8 @@ __device__ __forceinline__ void prefetch_rows_l2(const void* W, int row_bytes, i
             asm volatile("prefetch.global.L2 [%0];\n" ::"l"(static_cast<const char*>(W) + (size_t)e * row_bytes + off));
 }
 
-// The selection runs on 32-bit keys that order like the logits (sign-magnitude floats mapped to unsigned; -0 counts as
-// +0, a NaN ranks below every number), with two hardware warp reductions per selected expert: the largest key, then
-// the lowest index that holds it. Keys: 0 = no candidate (beyond E, or already selected), 1 = NaN, else the logit.
-// SLOTS = values per lane that can be occupied (2 covers 64 experts): this code runs once per token on the critical
-// path of a decode step, where every instruction is fetched cold, so the short form matters.
-__device__ __forceinline__ unsigned topk_key(float v) {
-    if (!(v == v)) return 1u;
-    const unsigned b = __float_as_uint(v + 0.f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float topk_value(unsigned key) {
-    if (key <= 1u) return key ? __uint_as_float(0x7fc00000u) : -INFINITY;
-    return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
-}
-// One selection step: returns the winner's index and key to every lane and retires it. With nothing left the result is
-// index 0 with key 0.
-template <int SLOTS>
-__device__ __forceinline__ void topk_step(unsigned (&key)[SLOTS], int lane, int& win_idx, unsigned& win_key) {
-    unsigned bk = 0u;
-#pragma unroll
-    for (int i = 0; i < SLOTS; ++i) bk = max(bk, key[i]);
-    win_key = __reduce_max_sync(0xffffffffu, bk);
-    unsigned cand = 0xffffffffu;
-#pragma unroll
-    for (int i = SLOTS - 1; i >= 0; --i) if (key[i] == win_key) cand = (unsigned)(lane + 32 * i);
-    const unsigned w = __reduce_min_sync(0xffffffffu, win_key ? cand : 0xffffffffu);
-    win_idx = (w == 0xffffffffu) ? 0 : (int)w;
-#pragma unroll
-    for (int i = 0; i < SLOTS; ++i) if (win_key && lane + 32 * i == win_idx) key[i] = 0u;
-}
-
+// Warp top-k over up to 256 values held 8 per lane (value j of lane l is element l + 32 j).
+// Order: value descending, index ascending. Lane 0 returns through out_idx / out_val (k <= 16).
 template <int SLOTS>
 __device__ __forceinline__ void warp_topk_n(const float (&v)[8], int E, int k, int lane, int* out_idx, float* out_val) {
     unsigned key[SLOTS];
@@ -947,10 +916,9 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
     if (threadIdx.x == 0) write_schedule(S.sched, s_tb, s_count, Etot, S.tc_min[0], S.tc_min[1]);
 }
 
-// S7 pooling: pooled[e] = mean_t score[t][e]; then the k_pred best pooled scores.
+// S7 pooling of per-token scores that the caller asked for: pooled[e] = mean_t score[t][e]; then the k_pred best.
 __global__ void __launch_bounds__(1024)
-k_pool(const float* __restrict__ ts, int T, int E, float* __restrict__ pooled, int32_t* __restrict__ ids, int k_pred,
-       int32_t* host_ids = nullptr, volatile uint32_t* host_flag = nullptr, uint32_t host_seq = 0) {
+k_pool(const float* __restrict__ ts, int T, int E, float* __restrict__ pooled, int32_t* __restrict__ ids, int k_pred) {
     __shared__ float s_pool[kMaxExperts];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int e = warp; e < E; e += 32) {
@@ -967,14 +935,8 @@ k_pool(const float* __restrict__ ts, int T, int E, float* __restrict__ pooled, i
         for (int i = 0; i < 8; ++i) v[i] = (lane + 32 * i < E) ? s_pool[lane + 32 * i] : -INFINITY;
         int oi[kMaxTopK]; float ov[kMaxTopK];
         warp_topk(v, E, k_pred, lane, oi, ov);
-        if (lane == 0) {
+        if (lane == 0)
             for (int j = 0; j < k_pred; ++j) ids[j] = oi[j];
-            if (host_ids != nullptr) {             // optional notification of a waiting host thread, as in the grouping kernel
-                for (int j = 0; j < k_pred; ++j) host_ids[j] = oi[j];
-                __threadfence_system();
-                *host_flag = host_seq;
-            }
-        }
     }
 }
 
@@ -1180,8 +1142,7 @@ mira_status launch_schedule(mira_ctx* ctx, int T, void* const* slots, const int3
 mira_status launch_pool(mira_ctx* ctx, const float* token_scores, int T, int E, float* pooled,
                         int32_t* ids, int k_pred, cudaStream_t st) {
     ProfScope ps(ctx, MIRA_K_POOL, st);
-    k_pool<<<1, 1024, 0, st>>>(token_scores, T, E, pooled, ids, k_pred, ids ? ctx->notify_ids : nullptr, ctx->notify_ids_flag,
-                               ctx->notify_seq);
+    k_pool<<<1, 1024, 0, st>>>(token_scores, T, E, pooled, ids, k_pred);
     ctx->launches += 1;
     MIRA_CUDA_OK(cudaGetLastError());
     return MIRA_OK;
@@ -1205,28 +1166,26 @@ mira_status set_route_attributes() {
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-// Scratch for the per-token scores of mira_predict_noalloc. It is part of the library image: every
-// GPU that loads libmira holds these 256 KB until the process exits, used or not.
-static __device__ __align__(256) float g_noalloc_token_scores[MIRA_NOALLOC_MAX_SCORES];
+// Scratch of mira_predict_noalloc: sums over token chunks (k_token_sums) of batches that need them. It is part of the
+// library image: every GPU that loads libmira holds these 256 KB until the process exits, used or not.
+static __device__ __align__(256) float g_noalloc_sums[MIRA_NOALLOC_MAX_SCORES];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mutex;
-float* g_noalloc_scores_addr[kMaxDevices];   // device address of the array above, per device (nullptr: not set up)
+float* g_noalloc_sums_addr[kMaxDevices];   // device address of the array above, per device (nullptr: not set up)
 
 // Once per device, with that device current: resolve the DEVICE address of the scratch array. In host
-// code the name `g_noalloc_token_scores` is only a host-side handle of the symbol; handing it to a
+// code the name `g_noalloc_sums` is only a host-side handle of the symbol; handing it to a
 // kernel would make the kernel touch the wrong memory.
 mira_status noalloc_setup(int dev, float** scratch) {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
-    if (g_noalloc_scores_addr[dev] == nullptr) {
+    if (g_noalloc_sums_addr[dev] == nullptr) {
         float* p = nullptr;
-        if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_noalloc_token_scores) != cudaSuccess || p == nullptr)
+        if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_noalloc_sums) != cudaSuccess || p == nullptr)
             return MIRA_ERR_CUDA;
-        if (cudaFuncSetAttribute(mira::k_scores, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
-            return MIRA_ERR_CUDA;
-        g_noalloc_scores_addr[dev] = p;
+        g_noalloc_sums_addr[dev] = p;
     }
-    *scratch = g_noalloc_scores_addr[dev];
+    *scratch = g_noalloc_sums_addr[dev];
     return MIRA_OK;
 }
 
@@ -1248,12 +1207,8 @@ extern "C" mira_status mira_predict_noalloc(const void* hidden, int32_t T, int32
     mira_status s = noalloc_setup(dev, &scratch);
     if (s != MIRA_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // every token score of this call is written before it is read, so nothing has to be cleared
-    k_scores<<<(T + kScoreTok - 1) / kScoreTok, kScoreThreads, scores_smem(hidden_size, n_experts), st>>>(
-        (const __nv_bfloat16*)hidden, T, hidden_size, (const __nv_bfloat16*)pred_w, pred_b, n_experts, scratch,
-        nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr);
-    k_pool<<<1, 1024, 0, st>>>(scratch, T, n_experts, out_expert_scores, out_topk_ids, out_topk_ids ? k_pred : 0);
-    MIRA_CUDA_OK(cudaGetLastError());
-    return MIRA_OK;
+    int launches = 0;          // every sum this call reads it has written before, so nothing has to be cleared
+    return launch_linear_head(hidden, T, hidden_size, pred_w, pred_b, n_experts, out_expert_scores, out_topk_ids,
+                              out_topk_ids ? k_pred : 0, scratch, nullptr, nullptr, 0, st, &launches);
 }
 
