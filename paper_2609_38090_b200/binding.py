@@ -159,13 +159,17 @@ def _check(code: int, where: str) -> None:
         raise MiraError(code, where)
 
 
+# Addresses and streams travel as plain integers (the prototypes above convert them): a ctypes object per argument and a
+# torch.cuda.Stream per call cost more host time than the library call of a small step.
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_current_device, _current_raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return _current_raw_stream(_current_device()) if stream is None else stream.cuda_stream
 
 
 class Mira:
@@ -243,25 +247,25 @@ class Mira:
     def predict(self, layer, hidden, pred_w, pred_b=None, k_pred=2, token_scores=False, stream=None, reuse=False):
         """reuse=True returns the same output tensors on every call with the same (T, k_pred, token_scores)."""
         T = hidden.shape[0]
-        key = ("predict", T, k_pred, bool(token_scores))
-        cache = self.__dict__.setdefault("_out_cache", {})
+        cache = self.__dict__.setdefault("_out_cache", {}) if reuse else None
+        key = ("predict", T, k_pred, bool(token_scores)) if reuse else None
         if reuse and key in cache:
             pooled, ts, ids = cache[key]
         else:
             pooled = torch.empty(self.E, dtype=torch.float32, device=self.device)
             ts = torch.empty((T, self.E), dtype=torch.float32, device=self.device) if token_scores else None
-            ids = torch.empty(max(k_pred, 1), dtype=torch.int32, device=self.device) if k_pred > 0 else None
+            ids = torch.empty(k_pred, dtype=torch.int32, device=self.device) if k_pred > 0 else None
             if reuse:
                 cache[key] = (pooled, ts, ids)
         _check(mira_predict(self._ctx, layer, _ptr(hidden), T, _ptr(pred_w), _ptr(pred_b), _ptr(pooled), _ptr(ts),
                             _ptr(ids), k_pred, _stream(stream)), "mira_predict")
-        return pooled, ts, (ids[:k_pred] if ids is not None else None)
+        return pooled, ts, ids
 
     def predict_mixture(self, layer, hidden, router_logits, count, k_top, head: dict, k_pred=2, stream=None):
         """MixtureHead on the by-products of mira_route. head: CUDA tensors wa_h, wa_l, wh_c, wh_t (bf16 matrices),
         g_h, g_l, g_c (bf16 vectors), b_a, b_h (fp32 vectors) and the float b_g. Returns (scores, probs, alpha, ids)."""
         T = hidden.shape[0]
-        hs = mira_mixture_head(*(head[n].data_ptr() for n in ("wa_h", "wa_l", "b_a", "wh_c", "wh_t", "b_h", "g_h", "g_l", "g_c")),
+        hs = mira_mixture_head(*[head[n].data_ptr() for n in ("wa_h", "wa_l", "b_a", "wh_c", "wh_t", "b_h", "g_h", "g_l", "g_c")],
                                float(head["b_g"]))
         scores = torch.empty(self.E, dtype=torch.float32, device=self.device)
         probs = torch.empty(self.E, dtype=torch.float32, device=self.device)
@@ -270,7 +274,7 @@ class Mira:
         _check(mira_predict_mixture(self._ctx, layer, _ptr(hidden), T, _ptr(router_logits), _ptr(count), k_top, C.byref(hs),
                                     _ptr(scores), _ptr(probs), _ptr(alpha), _ptr(ids), k_pred, _stream(stream)),
                "mira_predict_mixture")
-        return scores, probs, alpha, ids[:k_pred]
+        return scores, probs, alpha, ids if k_pred > 0 else ids[:k_pred]
 
     # S1-S6 ---------------------------------------------------------------------------------
     def _route_buffers(self, T, k, logits=True):
