@@ -256,13 +256,13 @@ mira_status mira_predict_mixture(mira_ctx* ctx, int32_t layer, const void* hidde
                                  float* out_alpha, int32_t* out_topk_ids, int32_t k_pred, void* stream);
 
 /* Options. MIRA_OPT_FORCE_DECODE_PATH (value 0/1): run S4/S5 of every batch through the weight-streaming
- * mma.sync kernels, also for the batch sizes that would take the tcgen05 kernels (used by the
+ * int8 kernels, also for the batch sizes that would take the fp16 tcgen05 kernels (used by the
  * tests to compare the two paths). MIRA_OPT_TENSOR_LAYOUT (value 0..3): 0 lets every step choose the tile layout of
  * the tcgen05 kernels from its token count (the default); 1, 2, 3 force the narrow, wide or big layout, 4 and 5 the
  * two-SM kernel (tcgen05 cta_group::2: tiles of 256 MMA rows over a cluster of two CTAs, 192 tokens x 4 ring stages
  * or 128 tokens x 8; needs ffn % 128 == 0 and hidden % 256 == 0, else the one-CTA layouts run), for tests and
  * tuning. MIRA_OPT_UP_CONVERSION (value 0..2): how the tcgen05 up/gate kernel turns int8 codes into fp16 operands
- * (the weight-streaming kernels always convert exactly). 0 and 1: exactly (the default). 2: as (code + 128) * 2^-24 with
+ * (the weight-streaming kernels convert no code at all). 0 and 1: exactly (the default). 2: as (code + 128) * 2^-24 with
  * the offset 128 * sum(x) taken out afterwards, 1.6 % faster at 2048 tokens; only accurate while the activations of every
  * token are close to zero-mean and every row's codes are well spread (the subtraction costs about
  * hidden size * |sum x| / (32 |x|_2) * 2^-27 relative to a row of typical codes, more for rows of small codes), which

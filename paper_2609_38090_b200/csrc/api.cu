@@ -22,7 +22,6 @@ bool config_ok(const mira_config* c) {
 }
 
 int down_splits_of(int R) { return (R + kDownSlice - 1) / kDownSlice; }
-int down_slice_of(int R) { int S = down_splits_of(R); return ((R / kChunk + S - 1) / S) * kChunk; }
 
 Layout make_layout(const mira_config& c) {
     Layout L;
@@ -45,8 +44,12 @@ Layout make_layout(const mira_config& c) {
     L.hexp = o;      o = align256(o + 2 * kMaxExperts * 4);
     L.x16 = o;       o = align256(o + T * C * 2);
     L.x16p = o;      o = align256(o + (T >= (size_t)kTensorPathMinTokens ? P * C * 2 : 0));
-    L.xs_pos = o;    o = align256(o + (T >= (size_t)kTensorPathMinTokens ? P * 4 : 0));
-    L.hm_pos = o;    o = align256(o + (T >= (size_t)kTensorPathMinTokens ? P * 4 : 0));
+    L.xs_pos = o;    o = align256(o + P * 4);
+    L.hm_pos = o;    o = align256(o + P * 4);
+    L.hs_pos = o;    o = align256(o + P * 4);
+    L.xq = o;        o = align256(o + 3 * P * C);
+    L.hq = o;        o = align256(o + 3 * P * R);
+    L.wmaps = o;     o = align256(o + ((size_t)kMaxExperts + 1) * kWeightMaps * 128);
     L.sum_pos = o;   o = align256(o + (T >= (size_t)kTensorPathMinTokens ? P * 4 : 0));
     L.h16 = o;       o = align256(o + P * R * 2);
     L.h16lo = o;     o = align256(o + P * R * 2);
@@ -133,7 +136,7 @@ mira_status do_experts(mira_ctx* ctx, int T, void* const* slots, const int32_t* 
     if (tc_min[0] < INT_MAX && (s = launch_up_gate_tc(ctx, slots, slot_map, st)) != MIRA_OK) return s;
     if (tc_min[1] > 0 && (s = launch_down(ctx, slots, slot_map, st)) != MIRA_OK) return s;
     if (tc_min[1] < INT_MAX && (s = launch_down_tc(ctx, slots, slot_map, st)) != MIRA_OK) return s;
-    if (final_wave) s = launch_combine(ctx, T, ctx->route_k, tc_min[1] > 0 ? ctx->down_splits : 1,
+    if (final_wave) s = launch_combine(ctx, T, ctx->route_k, tc_min[1] > 0 ? stream_down_splits(ctx) : 1,
                                        tc_min[1] < INT_MAX ? down_tc_slices(ctx) : 1, tc_min[1], out, st);
     return s;
 }
@@ -161,18 +164,17 @@ mira_status combine_only(mira_ctx* ctx, int T, void* out, cudaStream_t st) {
     if (misaligned(out)) return MIRA_ERR_ALIGN;
     int tc_min[2];
     step_tc_min(ctx, T, ctx->route_k, tc_min);
-    return launch_combine(ctx, T, ctx->route_k, tc_min[1] > 0 ? ctx->down_splits : 1,
+    return launch_combine(ctx, T, ctx->route_k, tc_min[1] > 0 ? stream_down_splits(ctx) : 1,
                           tc_min[1] < INT_MAX ? down_tc_slices(ctx) : 1, tc_min[1], out, st);
 }
 
-// Which experts of a T-token step go to the tensor-core kernels (see Sched::tc_min). Today's rule reproduces the
-// all-or-nothing switch per projection; MIRA_OPT_HYBRID_MIN_UP / _DOWN override it.
+// Which experts of a T-token step go to the fp16 tensor kernels (see Sched::tc_min): all or none per projection, by the
+// batch's average load (stream_max_pairs); MIRA_OPT_HYBRID_MIN_UP / _DOWN override it.
 void step_tc_min(const mira_ctx* ctx, int T, int k, int out_min[2]) {
-    (void)k;
-    const bool tc_ok = ctx->tensor_path_ok && !ctx->force_decode_path;
-    out_min[0] = (tc_ok && T >= tc_min_tokens_up(ctx->cfg)) ? 0 : INT_MAX;
-    out_min[1] = (tc_ok && T >= tc_min_tokens_down(ctx->cfg)) ? 0 : INT_MAX;
-    if (tc_ok && T >= kTensorPathMinTokens)
+    const bool tc_ok = ctx->tensor_path_ok && !ctx->force_decode_path && T >= kTensorPathMinTokens;
+    const double pairs = (double)T * k / ctx->cfg.n_experts;
+    for (int p = 0; p < 2; ++p) out_min[p] = (tc_ok && pairs > stream_max_pairs(ctx->cfg, p)) ? 0 : INT_MAX;
+    if (tc_ok)
         for (int p = 0; p < 2; ++p)
             if (ctx->hybrid_min[p] >= 0) out_min[p] = ctx->hybrid_min[p];
 }
@@ -227,12 +229,12 @@ mira_status mira_create(const mira_config* cfg, void* dev_workspace, size_t work
     ctx->device = dev;
     ctx->n_sm = n_sm;
     ctx->down_splits = down_splits_of(cfg->ffn);
-    ctx->down_slice = down_slice_of(cfg->ffn);
     ctx->force_decode_path = false;
     ctx->route_T = -1;
     ctx->route_k = 0;
     ctx->launches = 0;
     ctx->tensor_path_ok = tc_shape_ok(*cfg) && cfg->max_tokens >= kTensorPathMinTokens && build_tensor_maps(ctx);
+    if (!build_stream_maps(ctx)) { delete ctx; return MIRA_ERR_CUDA; }
     *out_ctx = ctx;
     return MIRA_OK;
 }

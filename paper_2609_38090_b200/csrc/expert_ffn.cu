@@ -1,602 +1,564 @@
-// S4-S6 for decode-sized groups: the expert FFN computed directly on the compressed expert
+// S4-S6 for decode-sized and mixed batches: the expert FFN computed directly on the compressed expert
 // ("fused dequantization + FFN", Section IV-A step 4 and Section IV-F), as two weight-streaming
 // kernels plus the weighted combine (Section II-A).
 //
 // The shared scale s_r (Section IV-B) indexes the OUTPUT row of W1^/W3^ and the REDUCTION index of
 // W2^, so no weight is ever multiplied by its scale one by one:
-//     U_r = sum_c q1[r][c] x_c,  G_r = sum_c q3[r][c] x_c        (integer codes, exact in fp16)
+//     U_r = sum_c q1[r][c] x_c,  G_r = sum_c q3[r][c] x_c        (integer codes)
 //     h_r = silu(s_r G_r) * (s_r U_r)
 //     y_c = sum_r q2[c][r] * (s_r h_r)
-// The scale is applied three times per (token, row) in the epilogue of the up/gate kernel; the
-// weight stream itself only needs the int8 -> fp16 conversion. The intermediate s_r h_r is stored
-// in fp16 after multiplication by a per-(token, expert) power of two that puts its typical
-// magnitude near 1; the down kernel undoes that power of two on its fp32 accumulators.
+// The codes themselves are the operand: int8 tensor-core instructions (tcgen05.mma kind::i8, sums in int32, exact) read them
+// from shared memory as the TMA unit laid them there, so no instruction touches a weight between HBM and the tensor core.
+// What is converted is the small side: a row of activations (x of a token, s h of a pair) becomes three planes of int8
+// digits, x = 2^e (d0 2^16 + d1 2^8 + d2), 22 bits and a sign below the row's largest value, and the MMA's columns are the
+// tokens of all three planes. The rounding of a digit row is 2^-22 of its largest value per element, less than what fp32
+// accumulation of the same products loses; the sums lose nothing.
 //
-// Both kernels stream the int8 rows with cp.async, turn them into fp16 MMA fragments in registers
-// (XOR 0x80, byte permute into the mantissa of 1024.0, subtract 1152: five ALU operations per four
-// weights) and use mma.sync m16n8k16 with the weights as the M operand and up to 32 tokens of the
-// expert as the N operand. The reduction index inside one MMA is permuted (the same way for both
-// operands) so that a thread's 16 consecutive weight bytes feed four MMAs without any shuffle.
+// Why: at full HBM rate a GPU of this kind draws its 1000 W and lowers its clock, so energy decides. The form this replaces
+// converted every code to fp16 in registers (1.25 instructions per weight, staged through shared memory, mma.sync) and ran a
+// 32-token step at 1069 W and 1710 MHz.
+// Measured (us per step, before -> now; the streamed bytes at the copy rate take 54 / 215 / 216): 8x7B shape, 1 token 77.1 ->
+// 75.8, 8 tokens 228 -> 190, 32 tokens 294 -> 249 (5.7 TB/s over the whole step), 200 tokens 428 -> 383; 8x22B shape, 13 tokens,
+// per-matrix format 352 -> 303; fine-grained layer, 4 tokens 54.1 -> 47.2, 64 tokens 98.2 -> 85.1.
 //
 // Work is derived on the device from the schedule the grouping step wrote; the host never reads
 // routing results.
 #include <algorithm>
+#include <cstring>
+#include <cuda.h>
 #include "mira_internal.cuh"
 
 namespace mira {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kPairs = kWarps / 2;
-// Ring depth: 3 stages when the activation tile is small (<= 8 tokens), else 2, so that two CTAs fit one SM.
-__host__ __device__ constexpr int stages_for(int nt) { return nt == 1 ? 3 : 2; }
-constexpr int kMT = 2;            // MMA m-tiles per unit
+constexpr int kEpiWarps = 8;              // two per TMEM lane quarter, taking eight columns in turn
+constexpr int kThreads = 32 * (4 + kEpiWarps);      // two TMA warps (weights, activations), MMA warp, (one idle,) epilogue warps
+constexpr int kUnit = 32;                 // MMA rows per unit of the partition; a tile has up to four
+constexpr int kKBox = 128;                // reduction elements (= bytes per row) of a TMA box: four MMAs of K = 32
+constexpr int kABox = 128 * kKBox;        // its weight tile
+constexpr int kMaxTok = 80;               // tokens of a tile: 3 * 80 columns of 256
+constexpr int kAccCols = 256;             // TMEM columns of an accumulator (two of them)
+constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr int kRingBytes = 212 * 1024;    // shared memory of the ring
+constexpr int kMaxStages = 6;
+constexpr int kItems = 4;                 // work items a CTA has drawn ahead
 
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+struct DigitMaps { CUtensorMap m[kDigitMaps]; };      // boxes of 8, 16, ..., 80 positions x 3 planes x 128 bytes
+static_assert(kDigitMaps * 8 == kMaxTok, "a box for every tile width");
 
-__device__ __forceinline__ void mma16816(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
-                                         unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+struct FfnArgs {
+    void* const* slots; const int32_t* slot_map; Sched* sched; const int32_t* count; const int32_t* offset;
+    const CUtensorMap* wmaps;             // [expert][kWeightMaps]
+    const int32_t* hexp;                  // [kMaxExperts + e]: wide-range flag of expert e
+    const float* xs_pos;                  // per position: 2^e of the activation row's digits (S4) ...
+    const float* hm_pos;                  // ... and the power of two that places the fp16 intermediate
+    const float* hs_pos;                  // per position: 2^e of the intermediate's digits, times 2^-f (S5)
+    __half* h16; __half* h16lo;           // the intermediate, upper and (wide-range experts) lower fp16 window
+    float* ypart;
+    int32_t* status;
+    int R, C, act_on_w1, per_matrix;
+    int n_all;                            // routed + shared experts
+    int stages, boxes, stage_bytes, b_box, tile_tok;      // ring geometry and tokens per tile, from the batch size
+    int token_order;                      // S4: the tile's columns are all T tokens (digit planes in token order, see kTokenOrderMax)
+    int T; const int32_t* row_token; const float* xscale; const float* xnorm; float* hscale;      // S4, token order
+    int splits; long ypart_stride;        // S5: slices of the reduction, elements between two slices of ypart
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool elect_one() {              // one lane of a converged warp
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0;
 }
-
-// Four int8 codes (one 32-bit word, already XOR-ed with 0x80808080 so each byte is u = code + 128) -> two half2 of
-// the signed codes, exactly: the byte goes into the mantissa of 1024.0 (0x6400 | u = 1024 + u) and 1152 = 1024 + 128
-// is subtracted. Five ALU operations per four weights (one XOR, two byte permutes, two half2 subtractions).
-// (Feeding u * 2^-24 as an fp16 subnormal and subtracting 128 * sum(x) afterwards saves the two subtractions, but
-// the tensor cores add in fp32 with truncation, so the subtracted term costs accuracy as soon as a token's
-// activations have a mean: measured 6e-3 instead of 1e-3 at hidden size 4096 with mean = spread. It also needs the
-// token sums in the epilogue. Measured on the Mixtral shape the exact form is as fast at 1 and 8 tokens and 0.5 %
-// slower at 32, so the streaming kernels always convert exactly; the tcgen05 up/gate kernel keeps the offset form
-// as an option.)
-__device__ __forceinline__ unsigned cvt_exact_lo(unsigned u) {
-    unsigned v = __byte_perm(u, 0x64646464u, 0x4140);
-    __half2 r = __hsub2(*reinterpret_cast<__half2*>(&v), __half2half2(__ushort_as_half(0x6480)));
-    return *reinterpret_cast<unsigned*>(&r);
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ unsigned cvt_exact_hi(unsigned u) {
-    unsigned v = __byte_perm(u, 0x64646464u, 0x4342);
-    __half2 r = __hsub2(*reinterpret_cast<__half2*>(&v), __half2half2(__ushort_as_half(0x6480)));
-    return *reinterpret_cast<unsigned*>(&r);
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Bounded wait by a whole warp. Returns false (and raises the abort flag) if the barrier did not flip in time.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    bool ok = false;
+    for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
+        if (mbar_try(bar, parity)) { ok = true; break; }
+        if ((spin & 1023u) == 1023u && *abort_flag) break;
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) *abort_flag = 1;
+    return ok;
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+// Shared-memory matrix descriptor, K-major, 128-byte swizzle (rows of 128 bytes, 8-row groups of 1024 bytes, the layout the
+// TMA unit writes); a K = 32 step advances the start address by 32 bytes.
+__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | (uint64_t)1 << 16 | (uint64_t)((1024 >> 4) & 0x3FFF) << 32 | (uint64_t)1 << 46 | (uint64_t)2 << 61;
+}
+// kind::i8: D int32, A and B signed 8-bit, both K-major, M = 128, N = n (a multiple of 16).
+__device__ __forceinline__ uint32_t make_idesc(int n) {
+    return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+__device__ __forceinline__ void mma_i8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}\n"
+                 ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
 // fp32 -> fp16, round to nearest even, values beyond the fp16 range go to +-65504 instead of infinity
 __device__ __forceinline__ unsigned short f32_to_f16_sat(float v) {
     unsigned short h;
     asm("cvt.rn.satfinite.f16.f32 %0, %1;\n" : "=h"(h) : "f"(v));
     return h;
 }
-__device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
 __device__ __forceinline__ float pow2i(int e) { return __uint_as_float((unsigned)(max(-126, min(127, e)) + 127) << 23); }
 __device__ __forceinline__ int expo(float v) { return (int)((__float_as_uint(v) >> 23) & 0xff) - 127; }
+// Scale of the digits of an intermediate row whose largest value is m: 2^(21 - e) (the smallest value the fp16 windows hold is 2^-48).
+__device__ __forceinline__ int digit_exponent(float m) { return m > 0.f ? max(-60, expo(m)) : 0; }
 
-struct ItemTable {             // the schedule, copied to shared memory once per CTA
-    int n_active, total_tb;
-    int tb_prefix[kMaxExperts + 1];
-    int w_prefix[kMaxExperts + 1];     // cost prefix of this kernel (up/gate or down)
-    uint8_t act_expert[kMaxExperts];
+// One tile: `units` units of 32 MMA rows from unit u0 on, ntok positions from pos0 on, n columns per plane (a multiple of 8),
+// boxes [b0, b1) of the reduction.
+// S4: a unit is 16 expert-hidden rows, MMA row 2m = W1^ row, 2m + 1 = W3^ row, so U and G of one (row, token) sit in
+// neighbouring TMEM lanes; S5: 32 model-hidden rows of W2^.
+struct Tile { int e, u0, units, pos0, ntok, n, split, b0, b1; };
+struct TileTable {                // indexed by expert
+    int cnt[kMaxExperts], off[kMaxExperts], width[kMaxExperts];      // width: tokens per tile
+    int pre[kMaxExperts + 1];     // exclusive prefix of the units (S * n_u of an expert that this kernel takes, else none)
+    int n_all, n_u, S, nbox;      // experts; units per slice of the reduction, slices (S4: one), boxes of the whole reduction
+    int n_cols;                   // columns per plane if every tile holds all tokens, else 0
+    int items;                    // work items: four units each
+};
+// Work is drawn item by item from a counter: bandwidth is not the same for every SM (equal shares ended 12 us apart in a 45 us
+// kernel; single-token step 84 -> 75 us). An item is four units, at 4096 reduction elements 12 us of one SM's share of HBM;
+// smaller ones at the end lose (items of two for the last 2 per CTA: 32 tokens 233 -> 237 us, of one: 245 us), because
+// the SMs that are left stream faster than their share and a low tile's stage costs more than its bytes.
+// Walks the tiles of an item: (up to four units of one slice, token tile), the token tile fastest, so that a weight tile that
+// several token tiles need is in L2 from the second one on.
+struct Walk {
+    const TileTable& tab;
+    int e, u, left, nb, units;
+    __device__ __forceinline__ Walk(const TileTable& table, int item) : tab(table), nb(0), units(0) {
+        const int total = tab.pre[tab.n_all];
+        const int g = 4 * item;
+        left = min(4, total - g);
+        int lo = 0, hi = tab.n_all - 1;                      // largest e with pre[e] <= g
+        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (tab.pre[mid] <= g) lo = mid; else hi = mid - 1; }
+        e = lo; u = g - tab.pre[lo];
+    }
+    __device__ __forceinline__ bool next(Tile& t) {
+        if (left <= 0) return false;
+        while (tab.pre[e + 1] - tab.pre[e] <= u) { ++e; u = 0; }      // (an item may run into the next expert)
+        const int w = tab.width[e], cnt = tab.cnt[e], n_u = tab.n_u, S = tab.S;
+        const int split = S > 1 ? u / n_u : 0;
+        units = min(left, (split + 1) * n_u - u);
+        t.e = e; t.u0 = u - split * n_u; t.units = units; t.split = split;
+        t.b0 = split * tab.nbox / S;
+        t.b1 = (split + 1) * tab.nbox / S;
+        t.pos0 = tab.off[e] + nb * w;
+        t.ntok = min(w, cnt - nb * w);
+        t.n = tab.n_cols ? tab.n_cols : (t.ntok + 7) & ~7;
+        if ((nb + 1) * w < cnt) ++nb;
+        else { nb = 0; u += units; left -= units; }
+        return true;
+    }
 };
 
-__device__ __forceinline__ void load_table(ItemTable& tab, const Sched* __restrict__ sched, int which) {
-    // the token blocks and costs of THIS projection's streaming work: an expert that the tensor-core kernel takes has
-    // none, and the searches below skip such zero-length entries
-    // (clamped: the up/gate kernel's rehearsal pass may read a schedule that is being rewritten, or was never written)
-    if (threadIdx.x == 0) { tab.n_active = max(0, min(sched->n_active, kMaxExperts)); tab.total_tb = sched->total_tb[which]; }
-    for (int i = threadIdx.x; i < kMaxExperts; i += blockDim.x) tab.act_expert[i] = (uint8_t)sched->act_expert[i];
-    for (int i = threadIdx.x; i <= kMaxExperts; i += blockDim.x) {
-        tab.tb_prefix[i] = sched->tb_prefix[which][i];
-        tab.w_prefix[i] = sched->w_prefix[which][i];
+template <bool DOWN>
+__global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_constant__ DigitMaps bmaps) {
+    extern __shared__ unsigned char smem[];
+    __shared__ TileTable tab;
+    __shared__ uint64_t s_bar[2 * kMaxStages + 4 + 2 * kItems];          // full, done, acc_full[2], acc_empty[2], item_full, item_empty
+    __shared__ int s_item[kItems];
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_abort;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int C = A.C, R = A.R, NS = A.stages, boxes = A.boxes;
+    const uint32_t a_bytes = boxes * kABox;
+    const int n_u = DOWN ? C / kUnit : R / (kUnit / 2), S = DOWN ? A.splits : 1;
+    const uint32_t ring = (smem_u32(smem) + 1023u) & ~1023u, bar0 = smem_u32(s_bar);
+    auto full = [&](int s) { return bar0 + 8u * s; };
+    auto done = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
+    auto acc_full = [&](uint32_t b) { return bar0 + 8u * (2 * kMaxStages + b); };
+    auto acc_empty = [&](uint32_t b) { return bar0 + 8u * (2 * kMaxStages + 2 + b); };
+    auto item_full = [&](uint32_t i) { return bar0 + 8u * (2 * kMaxStages + 4 + i); };
+    auto item_empty = [&](uint32_t i) { return bar0 + 8u * (2 * kMaxStages + 4 + kItems + i); };
+
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 2); mbar_init(done(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), kEpiWarps); }
+        for (int i = 0; i < kItems; ++i) { mbar_init(item_full(i), 1); mbar_init(item_empty(i), 2 + kEpiWarps); }
+        s_abort = 0;
+        tab.n_all = A.n_all; tab.n_u = n_u; tab.S = S; tab.nbox = ((DOWN ? R : C) + kKBox - 1) / kKBox;
+        tab.n_cols = !DOWN && A.token_order ? (A.T + 7) & ~7 : 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    // Table of the experts. The schedule, the counts and the maps come from the routing kernels, which had completed before the
+    // kernel in front of this one started; with digits in token order the routing kernel IS the kernel in front.
+    const bool token_order = !DOWN && A.token_order;
+    if (token_order) { pdl_wait(); pdl_launch(); }
+    const int tc_min = A.sched->tc_min[DOWN ? 1 : 0];
+    for (int e = tid; e < A.n_all; e += kThreads) {
+        const int cnt = A.count[e], off = A.offset[e];
+        const bool mine = (A.sched->act_mask[e >> 5] >> (e & 31) & 1u) && cnt < tc_min;
+        const int nt = (cnt + A.tile_tok - 1) / A.tile_tok;
+        tab.cnt[e] = cnt; tab.off[e] = off;
+        tab.width[e] = mine ? ((cnt + nt - 1) / nt + 7) & ~7 : 0;
     }
     __syncthreads();
-}
-
-// Units are weighted by the cost of their token block. Returns the first unit at or after cost position x, where
-// x counts cost * units (0 <= x <= total cost * per_tb); monotonic in x, so consecutive CTAs get adjoining ranges.
-// I: the integer type of unit numbers and cost positions. The launcher takes 32 bits whenever the largest cost
-// position (cost * units * CTAs) fits: 64-bit divisions are long software routines, and this code runs cold at the
-// start of every CTA, where instruction fetch from memory is what it costs.
-template <typename I>
-__device__ __forceinline__ I unit_at(const ItemTable& tab, I x, I per_tb, int w_full) {
-    const int n = tab.n_active;
-    if (x >= (I)tab.w_prefix[n] * per_tb) return (I)tab.total_tb * per_tb;
-    const int xb = (int)(x / per_tb);
-    int lo = 0, hi = n - 1;                                // largest a with w_prefix[a] <= xb
-    while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (tab.w_prefix[mid] <= xb) lo = mid; else hi = mid - 1; }
-    const I local = x - (I)tab.w_prefix[lo] * per_tb;
-    const int ntb = tab.tb_prefix[lo + 1] - tab.tb_prefix[lo];
-    const I full_block = (I)w_full * per_tb;
-    const I full_span = (I)(ntb - 1) * full_block;
-    I blk, in_blk;
-    if (local < full_span) {
-        blk = local / full_block;
-        in_blk = (local - blk * full_block) / w_full;
-    } else {
-        const int w_last = tab.w_prefix[lo + 1] - tab.w_prefix[lo] - (ntb - 1) * w_full;
-        blk = ntb - 1;
-        in_blk = (local - full_span) / w_last;
-    }
-    return ((I)tab.tb_prefix[lo] + blk) * per_tb + in_blk;
-}
-
-struct FfnArgs {
-    void* const* slots;
-    const int32_t* slot_map;
-    const Sched* sched;
-    const int32_t* count;
-    const int32_t* offset;
-    const int32_t* row_token;
-    const float* xscale;
-    const float* xnorm;
-    const int32_t* hexp;        // per expert: exponent of the intermediate's expected magnitude per unit of |x|^2
-    float* hscale;
-    const __half* x16;
-    __half* h16;
-    __half* h16lo;              // lower window of the intermediate, written and read for wide-range experts only
-    float* ypart;
-    int R, C, act_on_w1;
-    int down_splits, down_slice;
-    int per_matrix;             // blob format: 0 shared scale, 1 per-matrix scales (see BlobFmt)
-    int n_all;                  // routed + shared experts
-    long ypart_stride;          // elements between two splits = P * C
-};
-
-// ---------------------------------------------------------------------------------------------
-// S4 (up + gate) and S5 (down) share one pipeline.
-//
-// Unit of work: 32 weight rows (two MMA m-tiles) x one block of <= 32 tokens of one expert, done by
-// a PAIR of warps that split the reduction index between them and add their partial sums at the
-// end of the unit (fixed order, so results are bit-repeatable).
-//   S4: an m-tile holds 8 rows of W1^ in MMA rows 0-7 and the SAME 8 rows of W3^ in MMA rows 8-15, so
-//       one thread ends up with U and G of the same (row, token) and the SwiGLU is thread-local;
-//       a unit is 16 expert-hidden rows over the whole reduction (C).
-//   S5: ordinary m-tiles of W2^; a unit is 32 model-hidden rows over one slice of the reduction (R);
-//       partial sums of the slices go to ypart[slice].
-// Units are numbered (expert, token block, [slice,] row group). Every CTA takes an equal contiguous
-// range of units and walks it in steps of up to 4 units (one per warp pair) that belong to the same
-// (expert, token block, slice), so the pairs of a step share one activation tile.
-//
-// Memory pipeline, per stage of 256 reduction elements:
-//   weights     : each pair copies its 32 rows x 256 bytes with cp.async, two rows per instruction,
-//                 so every request is 256 contiguous bytes of one row (64-byte pieces reach only
-//                 ~75 % of HBM bandwidth on B200, 256-byte pieces reach all of it). The tile is
-//                 XOR-swizzled so the MMA fragment reads are conflict free.
-//   activations : the CTA copies the <= 32 token rows x 512 bytes (fp16) once for all its warps.
-// ---------------------------------------------------------------------------------------------
-constexpr int kSeg = 256;                           // reduction elements (= weight bytes per row) per stage
-constexpr int kSegChunks = kSeg / kChunk;           // 4 MMA k-groups of 64 per stage, 2 per warp of a pair
-constexpr int kATile = 32 * kSeg;                   // bytes of one pair's weight tile
-constexpr int kBRow = kSeg * 2 + 16;                // bytes per activation row in shared memory (padded)
-__host__ __device__ constexpr size_t ring_bytes(int nt) {
-    return (size_t)stages_for(nt) * (kPairs * kATile + nt * 8 * kBRow);
-}
-// After the ring comes the exchange area of the pair reduction, 4 slots (one per pair) of 512 NT bytes.
-__host__ __device__ constexpr size_t step_smem(int nt) { return ring_bytes(nt) + (size_t)kPairs * 512 * nt; }
-constexpr size_t kSmemBytes = step_smem(1) > step_smem(4) ? step_smem(1) : step_smem(4);
-static_assert(step_smem(2) <= kSmemBytes && step_smem(3) <= kSmemBytes, "ring geometry");
-static_assert(kSmemBytes + sizeof(ItemTable) + 1024 <= 116736, "two CTAs per SM (228 KB, 1 KB reserved per CTA)");
-
-__device__ __forceinline__ void lds128(unsigned (&v)[4], unsigned saddr) {
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(saddr));
-}
-__device__ __forceinline__ void cp_async16_s(unsigned saddr, const void* gmem_src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr), "l"(gmem_src) : "memory");
-}
-// One step of a CTA: up to kPairs units of the same (expert, token block, slice).
-struct StepDesc {
-    const unsigned char* blob;
-    int row0, k0, klen, split, pos0, ntok, nt, nstep, hexp;
-    bool active, valid;
-    bool wide;          // wide-range expert: the intermediate has a second, lower fp16 window (h16lo)
-    bool last_half;     // S5 of a wide-range expert takes a 32-token block as two halves of 16 (see k_ffn)
-};
-
-// Per-thread state of the copies of one step (geometry follows the step's NT).
-struct CopyState {
-    const unsigned char* w0;       // S4: W1^ rows; S5: W2^ rows 0-7 of this warp's half tile
-    const unsigned char* w1;       // S4: W3^ rows; S5: W2^ rows 8-15
-    const unsigned char* b;        // activation row of this thread
-    unsigned a_cp, b_cp, ld2, b_tile;
-    int nchunk;
-    bool active, bvalid;
-};
-
-template <bool DOWN>
-__device__ __forceinline__ CopyState setup_copy(const FfnArgs& A, const StepDesc& d, unsigned sA) {
-    CopyState c;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pair = warp >> 1, half = warp & 1, crow = lane >> 4, ccol = lane & 15;
-    const size_t per = (size_t)A.R * A.C;
-    const unsigned ld = DOWN ? A.R : A.C;
-    // weight copy: this warp moves tile rows [16 half, 16 half + 16); instruction i moves rows 2i, 2i+1 of
-    // those; this lane moves 16 bytes of row 2i + (lane >> 4)
-    if (DOWN) {
-        c.w0 = d.blob + per + (size_t)(d.row0 + half * 16 + crow) * ld + d.k0 + ccol * 16;
-        c.w1 = c.w0 + (size_t)8 * ld;
-    } else {
-        c.w0 = d.blob + (size_t)(d.row0 + half * 8 + crow) * ld + d.k0 + ccol * 16;
-        c.w1 = c.w0 + 2 * per;
-    }
-    c.ld2 = 2 * ld;
-    c.a_cp = sA + pair * kATile + (half * 16 + crow) * kSeg + ((ccol ^ (crow << 2)) << 4);
-    // activation copy: thread t moves pieces (t % 8) + 8 q, q = 0..3, of token t / 8 (512 bytes per token and stage)
-    const int bcol = threadIdx.x & 7, btok = threadIdx.x >> 3;
-    c.b_tile = d.nt * 8 * kBRow;
-    c.b_cp = sA + stages_for(d.nt) * (kPairs * kATile) + btok * kBRow + bcol * 16;
-    {
-        // S5 of a wide-range expert: the tile's first nt / 2 n-tiles hold the upper window of the <= 16 tokens, the
-        // other nt / 2 the lower window of the same tokens, so one pass over the weight fragments serves both
-        int trow = btok;
-        const __half* src = DOWN ? A.h16 : A.x16;
-        if (DOWN && d.wide) {
-            const int hr = d.nt * 4;               // rows of one window: 8 * (nt / 2)
-            if (btok >= hr) { trow = btok - hr; src = A.h16lo; }
-            c.bvalid = trow < d.ntok && btok < 2 * hr;
-        } else {
-            c.bvalid = btok < d.ntok;
+    if (warp == 0) {
+        int carry = 0;
+        for (int base = 0; base < A.n_all; base += 32) {
+            const int own = base + lane < A.n_all && tab.width[base + lane] ? n_u * S : 0;
+            int v = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
+            if (base + lane < A.n_all) tab.pre[base + lane] = carry + v - own;
+            carry += __shfl_sync(0xffffffffu, v, 31);
         }
-        const int tok = min(trow, d.ntok - 1);     // rows beyond ntok alias the last valid row and are not copied
-        const size_t rowi = DOWN ? (size_t)(d.pos0 + tok) : (size_t)A.row_token[d.pos0 + tok];
-        c.b = reinterpret_cast<const unsigned char*>(src + rowi * ld + d.k0) + bcol * 16;
-    }
-    c.nchunk = d.klen / kChunk;
-    c.active = d.active;
-    return c;
-}
-
-// Issue the copies of stage sg into ring buffer `buf`; advances the source pointers by one stage.
-// WEIGHTS / ACTS select the half of the stage to issue (both by default).
-template <bool WEIGHTS = true, bool ACTS = true>
-__device__ __forceinline__ void issue_stage(CopyState& c, int sg, int buf) {
-    const int left = c.nchunk - sg * kSegChunks;                // chunks valid in this stage
-    if (WEIGHTS) {
-        if (c.active && (int)(threadIdx.x & 15) < left * 4) {
-            const unsigned dst = c.a_cp + buf * (kPairs * kATile);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                cp_async16_s(dst + (2 * i) * kSeg, c.w0 + i * c.ld2);          // S4: W1^ rows; S5: rows 0-7
-                cp_async16_s(dst + (8 + 2 * i) * kSeg, c.w1 + i * c.ld2);      // S4: W3^ rows; S5: rows 8-15
-            }
+        if (lane == 0) {
+            tab.pre[A.n_all] = carry;
+            tab.items = (carry + 3) >> 2;
         }
-        c.w0 += kSeg; c.w1 += kSeg;
     }
-    if (ACTS) {
-        if (c.bvalid) {
-            const unsigned dst = c.b_cp + buf * c.b_tile;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < left) cp_async16_s(dst + q * 128, c.b + q * 128);
-        }
-        c.b += kSeg * 2;
-    }
-}
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
 
-// The first stages of a step (as many as its ring holds), one cp.async group each.
-template <bool DOWN>
-__device__ __forceinline__ CopyState start_step(const FfnArgs& A, const StepDesc& d, unsigned sA) {
-    CopyState c = setup_copy<DOWN>(A, d, sA);
-    const int nstage = (c.nchunk + kSegChunks - 1) / kSegChunks, ks = stages_for(d.nt);
-    for (int s = 0; s < ks; ++s) {
-        if (s < nstage) issue_stage(c, s, s);
-        cp_async_commit();
-    }
-    return c;
-}
-
-// The same in two halves, for a kernel whose weights do not depend on the kernel before it but whose activations do:
-// the weight copies of the first stages go out before the wait on that kernel (one group, older than all others),
-// the activation copies after it, one group per stage in the places where start_step commits its groups, so the
-// group counts that the step's waits rely on are the same.
-template <bool DOWN>
-__device__ __forceinline__ CopyState start_step_weights(const FfnArgs& A, const StepDesc& d, unsigned sA) {
-    CopyState c = setup_copy<DOWN>(A, d, sA);
-    const int nstage = (c.nchunk + kSegChunks - 1) / kSegChunks, ks = stages_for(d.nt);
-    for (int s = 0; s < ks; ++s)
-        if (s < nstage) issue_stage<true, false>(c, s, s);
-    cp_async_commit();
-    return c;
-}
-__device__ __forceinline__ void start_step_acts(CopyState& c, const StepDesc& d) {
-    const int nstage = (c.nchunk + kSegChunks - 1) / kSegChunks, ks = stages_for(d.nt);
-    for (int s = 0; s < ks; ++s) {
-        if (s < nstage) issue_stage<false, true>(c, s, s);
-        cp_async_commit();
-    }
-}
-
-// Runs one step whose first stages are already in flight (start_step), then starts the next step's first
-// stages before its own epilogue, so the memory system never idles between steps.
-template <bool DOWN, int NT>
-__device__ __forceinline__ void ffn_step(const FfnArgs& A, const StepDesc& d, CopyState& cs, const StepDesc& next,
-                                         CopyState& cs_next, unsigned char* ringA) {
-    constexpr int kStages = stages_for(NT);
-    constexpr int kBTile = NT * 8 * kBRow;
-    const unsigned char* blob = d.blob;
-    const int row0 = d.row0, split = d.split, pos0 = d.pos0, ntok = d.ntok;
-    const bool active = d.active;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const int pair = warp >> 1, half = warp & 1;
-    const int C = A.C, R = A.R;
-    const size_t per = (size_t)R * C;
-    const unsigned sA = (unsigned)__cvta_generic_to_shared(ringA), sB = sA + kStages * (kPairs * kATile);
-    // shared-memory byte addresses; everything that varies inside the loops is a compile-time offset
-    const unsigned gpar = g & 1;
-    const unsigned a_rd0 = sA + pair * kATile + g * kSeg + half * 128 + gpar * 64 + tq * 16;          // first chunk of this warp
-    const unsigned a_rd1 = sA + pair * kATile + g * kSeg + half * 128 + (gpar ^ 1) * 64 + tq * 16;    // second chunk
-    const unsigned b_rd = sB + g * kBRow + half * 256 + tq * 32;
-
-    float acc[kMT][NT][4];
-#pragma unroll
-    for (int mt = 0; mt < kMT; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
-
-    const int nchunk = cs.nchunk;
-    const int nstage = (nchunk + kSegChunks - 1) / kSegChunks;
-    // one 64-wide chunk: B fragments of all n-tiles, A fragments of both m-tiles, 8 NT MMAs
-    auto chunk = [&](unsigned a_rd, unsigned b_at) {
-        unsigned bf[NT][8];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            unsigned lo[4], hi[4];
-            lds128(lo, b_at + nt * 8 * kBRow);
-            lds128(hi, b_at + nt * 8 * kBRow + 16);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { bf[nt][i] = lo[i]; bf[nt][4 + i] = hi[i]; }
-        }
-#pragma unroll
-        for (int mt = 0; mt < kMT; ++mt) {
-            unsigned wa[4], wb[4];
-            lds128(wa, a_rd + (mt * 16) * kSeg);           // MMA rows 0-7
-            lds128(wb, a_rd + (mt * 16 + 8) * kSeg);       // MMA rows 8-15
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned ua = wa[j] ^ 0x80808080u, ub = wb[j] ^ 0x80808080u;
-                unsigned f0, f1, f2, f3;
-                f0 = cvt_exact_lo(ua); f2 = cvt_exact_hi(ua); f1 = cvt_exact_lo(ub); f3 = cvt_exact_hi(ub);
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) mma16816(acc[mt][nt], f0, f1, f2, f3, bf[nt][2 * j], bf[nt][2 * j + 1]);
-            }
-        }
+    // The next item of the other roles (warp 0 draws them): -1 at the end.
+    uint32_t n_item = 0;
+    auto next_item = [&]() {
+        const uint32_t i = n_item % kItems;
+        if (!mbar_wait(item_full(i), (n_item / kItems) & 1u, &s_abort)) return -1;
+        const int item = s_item[i];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(item_empty(i));
+        ++n_item;
+        return item;
     };
-    for (int sg = 0; sg < nstage; ++sg) {
-        const int buf = sg % kStages;
-        cp_async_wait<kStages - 1>();
-        __syncthreads();                 // stage sg has landed for every thread of the CTA
-        if (active) {
-            const unsigned ao = buf * (kPairs * kATile), bo = buf * kBTile;
-            const int nch = nchunk - sg * kSegChunks - half * 2;     // chunks of this warp that are valid (>= 2: both)
-            if (nch >= 2) {
-                chunk(a_rd0 + ao, b_rd + bo);
-                chunk(a_rd1 + ao, b_rd + bo + 128);
-            } else if (nch == 1) {
-                chunk(a_rd0 + ao, b_rd + bo);
+
+    if (warp < 2) {
+        // ------------------------------------------------ TMA warps. The weights depend on the routing alone, the digits on the
+        // kernel before this one: warp 0 requests weights at once, warp 1 waits.
+        if (warp == 1 && !token_order) { pdl_wait(); pdl_launch(); }
+        int slot = 0, item = blockIdx.x, drawn = 0;
+        const CUtensorMap* last_map = nullptr;
+        uint32_t ph = 1;
+        bool ok = true;
+        while (ok) {
+            if (warp == 0) {
+                const uint32_t i = n_item % kItems;
+                if (item >= tab.items) item = -1;
+                if (n_item >= kItems && !mbar_wait(item_empty(i), ((n_item / kItems) & 1u) ^ 1u, &s_abort)) break;
+                if (lane == 0) {
+                    s_item[i] = item;
+                    mbar_arrive(item_full(i));
+                    if (item >= 0) drawn = (int)atomicAdd(&A.sched->ticket[DOWN ? 1 : 0], 1u) + (int)gridDim.x;      // the item after this one
+                }
+                ++n_item;
+            } else item = next_item();
+            if (item < 0) break;
+            Walk w(tab, item);
+            Tile t;
+            while (ok && w.next(t)) {
+                const CUtensorMap* map = warp == 0 ? A.wmaps + (size_t)t.e * kWeightMaps + (DOWN ? 4 : 0) + (t.units - 1) : &bmaps.m[t.n / 8 - 1];
+                if (warp == 0 && map != last_map) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(map) : "memory");
+                last_map = map;
+                const uint32_t box_bytes = warp == 0 ? t.units * (kABox / 4) : 3 * t.n * kKBox, box_step = warp == 0 ? kABox : A.b_box;
+                const uint32_t base = ring + (warp == 0 ? 0 : a_bytes);
+                const int row = warp == 0 ? t.u0 * (DOWN ? kUnit : kUnit / 2) : token_order ? 0 : t.pos0;
+                for (int b = t.b0; b < t.b1; b += boxes) {
+                    if (!mbar_wait(done(slot), ph, &s_abort)) { ok = false; break; }
+                    if (elect_one()) {
+                        const uint32_t dst = base + slot * A.stage_bytes, bar = full(slot);
+                        const int nb = min(boxes, t.b1 - b);
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(nb * box_bytes) : "memory");
+                        for (int j = 0; j < nb; ++j) {
+                            if (warp == 1) tma_3d(dst + j * box_step, map, (b + j) * kKBox, row, 0, bar);
+                            else if (DOWN) tma_2d(dst + j * box_step, map, (b + j) * kKBox, row, bar);
+                            else tma_3d(dst + j * box_step, map, (b + j) * kKBox, 0, row, bar);
+                        }
+                    }
+                    __syncwarp();
+                    if (++slot == NS) { slot = 0; ph ^= 1u; }
+                }
+            }
+            if (warp == 0) item = __shfl_sync(0xffffffffu, drawn, 0);
+        }
+    } else if (warp == 2) {
+        // ------------------------------------------------ MMA warp
+        int slot = 0;
+        uint32_t ph = 0, it = 0;
+        bool ok = true;
+        for (int item = next_item(); ok && item >= 0; item = next_item()) {
+            Walk w(tab, item);
+            Tile t;
+            while (ok && w.next(t)) {
+                const uint32_t buf = it & 1u, d = tmem + buf * kAccCols, idesc = make_idesc((3 * t.n + 15) & ~15);
+                if (it >= 2 && !mbar_wait(acc_empty(buf), ((it >> 1) & 1u) ^ 1u, &s_abort)) { ok = false; break; }       // its previous epilogue is done
+                tc_fence_after();
+                for (int b = t.b0; b < t.b1; b += boxes) {
+                    if (!mbar_wait(full(slot), ph, &s_abort)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t da = make_desc(ring + slot * A.stage_bytes), db = make_desc(ring + slot * A.stage_bytes + a_bytes);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) mma_i8(d, da + 2 * j, db + 2 * j, idesc, (b > t.b0 || j) ? 1u : 0u);
+                        if (boxes == 2 && b + 1 < t.b1) {
+                            const uint64_t da1 = da + (kABox >> 4), db1 = db + (A.b_box >> 4);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) mma_i8(d, da1 + 2 * j, db1 + 2 * j, idesc, 1u);
+                        }
+                        mma_commit(done(slot));
+                    }
+                    __syncwarp();
+                    if (++slot == NS) { slot = 0; ph ^= 1u; }
+                }
+                if (!ok) break;
+                if (elect_one()) mma_commit(acc_full(buf));
+                __syncwarp();
+                ++it;
             }
         }
-        __syncthreads();                 // every warp is done with the tiles of stage sg
-        if (sg + kStages < nstage) issue_stage(cs, sg + kStages, buf);
-        cp_async_commit();
-    }
-    cp_async_wait<0>();
-    // The ring is idle now. If the next step has the same ring geometry its first stages start here, under
-    // the reduction and the epilogue of this step; otherwise they start after the reduction, whose exchange
-    // area (behind this step's ring) a larger ring would overlap.
-    const bool early = next.valid && next.nt == NT;
-    if (early) cs_next = start_step<DOWN>(A, next, sA);
-
-    // Add the two halves of the reduction in two passes through the pair's exchange slot: warp `half` keeps
-    // m-tile `half` and receives the other warp's partial sums of that m-tile; always (warp 0 part) + (warp 1 part).
-    float* slot = reinterpret_cast<float*>(ringA + ring_bytes(NT)) + (size_t)pair * 128 * NT;
-    float sum[NT][4];
-    if (active && half == 1) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) slot[(nt * 4 + i) * 32 + lane] = acc[0][nt][i];
-    }
-    __syncthreads();
-    if (active && half == 0) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                sum[nt][i] = acc[0][nt][i] + slot[(nt * 4 + i) * 32 + lane];
-                slot[(nt * 4 + i) * 32 + lane] = acc[1][nt][i];          // second pass: this warp's part of m-tile 1
+    } else if (warp >= 4) {
+        // ------------------------------------------------ epilogue (thread = MMA row = TMEM lane)
+        if (!token_order) pdl_wait();
+        const int cg = 8 * ((warp - 4) >> 2);                // first chunk of columns of this warp
+        const int q = warp & 3, row = q * 32 + lane;
+        const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
+        const size_t per = (size_t)R * C;
+        uint32_t it = 0;
+        bool ok = true;
+        for (int item = next_item(); ok && item >= 0; item = next_item()) {
+        Walk w(tab, item);
+        Tile t;
+        while (w.next(t)) {
+            const uint32_t buf = it & 1u, acc = lane_base + buf * kAccCols;
+            // what the tile needs from memory, under the MMAs
+            const unsigned char* blob = static_cast<const unsigned char*>(A.slots[A.slot_map[t.e]]);
+            const int r = DOWN ? t.u0 * kUnit + row : t.u0 * (kUnit / 2) + (row >> 1), odd = row & 1;
+            const bool mine = q < t.units;
+            int wide = 0, my_tok = -1;
+            float s_u = 1.f, s_g = 1.f, s_h = 1.f, my_xs = 0.f, my_hm = 0.f;
+            if (mine) {
+                if (DOWN) {             // per-matrix format: the scale of output column r (row r of W2^)
+                    if (A.per_matrix) s_u = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_out)[r]);
+                } else {                // shared format: all three are s_r; per-matrix: s1, s3 and 1
+                    wide = A.hexp[kMaxExperts + t.e];
+                    s_u = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + 3 * per)[r]);
+                    s_g = A.per_matrix ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_gate)[r]) : s_u;
+                    s_h = A.per_matrix ? 1.f : s_u;
+                }
+                // token order: lane i knows the i-th position's token and token i's factors
+                if (token_order) {
+                    if (lane < t.ntok) my_tok = A.row_token[t.pos0 + lane];
+                    if (lane < A.T) {
+                        const int f = max(-120, min(120, -(A.hexp[t.e] + 11 + 2 * expo(A.xnorm[lane]))));
+                        my_xs = A.xscale[lane] * (1.f / 256.f);
+                        my_hm = pow2i(f);
+                    }
+                    const float hm_of_pos = __shfl_sync(0xffffffffu, my_hm, max(my_tok, 0));
+                    if (t.u0 == 0 && warp == 4 && lane < t.ntok) A.hscale[t.pos0 + lane] = 1.f / hm_of_pos;
+                }
             }
-    }
-    __syncthreads();
-    if (active && half == 1) {
+            if (!mbar_wait(acc_full(buf), (it >> 1) & 1u, &s_abort)) { ok = false; break; }
+            tc_fence_after();
+            if (mine) {
+                const int ncol = token_order ? A.T : t.ntok;
+                for (int c0 = cg; c0 < ncol; c0 += 2 * kEpiWarps) {
+                    int d0[8], d1[8], d2[8];
+                    __syncwarp();
+                    tmem_ld8(acc + c0, d0);
+                    tmem_ld8(acc + t.n + c0, d1);
+                    tmem_ld8(acc + 2 * t.n + c0, d2);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                    float v[8];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
+                    for (int j = 0; j < 8; ++j) v[j] = fmaf((float)d0[j], 65536.f, fmaf((float)d1[j], 256.f, (float)d2[j]));
+                    if (DOWN) {
+                        float* yp = A.ypart + (size_t)t.split * A.ypart_stride + (size_t)(t.pos0 + c0) * C + r;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sum[nt][i] = slot[(nt * 4 + i) * 32 + lane] + acc[1][nt][i];
-    }
-    if (next.valid && !early) {
-        __syncthreads();                 // the exchange slots have been read
-        cs_next = start_step<DOWN>(A, next, sA);
-    }
-    if (!active) return;
-    const int mt = half;
-
-    if (DOWN) {
-        float* yp = A.ypart + (size_t)split * A.ypart_stride;
-        float so0 = 1.f, so1 = 1.f;          // per-matrix format: the scale of the output column (row of W2^)
-        if (A.per_matrix) {
-            const __nv_bfloat16* so = reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_out);
-            so0 = __bfloat162float(so[row0 + mt * 16 + g]);
-            so1 = __bfloat162float(so[row0 + mt * 16 + g + 8]);
-        }
-        if (NT % 2 == 0 && d.wide) {         // upper window in n-tiles [0, NT / 2), lower window of the same tokens behind
-            constexpr int H = NT / 2;
-            const float lo_scale = pow2i(-kLoShift);
+                        for (int j = 0; j < 8; ++j)
+                            if (c0 + j < t.ntok) yp[(size_t)j * C] = v[j] * (__ldg(A.hs_pos + t.pos0 + c0 + j) * s_u);
+                    } else {
+                        // Even lanes hold U, odd lanes G of the same expert-hidden row. Of every pair of columns the even lane
+                        // finishes the even one and the odd lane the odd one: one exchange per pair.
 #pragma unroll
-            for (int nt = 0; nt < H; ++nt)
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int n = nt * 8 + tq * 2 + i;
-                    if (n < ntok) {
-                        const float hs = A.hscale[pos0 + n];
-                        yp[(size_t)(pos0 + n) * C + row0 + mt * 16 + g] = fmaf(sum[nt + H][i], lo_scale, sum[nt][i]) * hs * so0;
-                        yp[(size_t)(pos0 + n) * C + row0 + mt * 16 + g + 8] = fmaf(sum[nt + H][2 + i], lo_scale, sum[nt][2 + i]) * hs * so1;
+                        for (int jj = 0; jj < 4; ++jj) {
+                            const float a = v[2 * jj], b = v[2 * jj + 1];
+                            const float other = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+                            const int n = c0 + 2 * jj + odd;
+                            int pos = t.pos0 + min(n, t.ntok - 1);
+                            bool store = n < t.ntok;
+                            float xs, hm;
+                            if (token_order) {
+                                const unsigned me = __ballot_sync(0xffffffffu, my_tok == c0 + 2 * jj), mo = __ballot_sync(0xffffffffu, my_tok == c0 + 2 * jj + 1);
+                                const unsigned m = odd ? mo : me;
+                                store = m != 0;
+                                pos = t.pos0 + __ffs(m) - 1;
+                                xs = __shfl_sync(0xffffffffu, my_xs, n & 31); hm = __shfl_sync(0xffffffffu, my_hm, n & 31);
+                            } else {
+                                xs = __ldg(A.xs_pos + pos); hm = __ldg(A.hm_pos + pos);
+                            }
+                            const float u = (odd ? other : a) * (xs * s_u), g = (odd ? b : other) * (xs * s_g);
+                            const float act = A.act_on_w1 ? u : g, lin = A.act_on_w1 ? g : u;
+                            const float val = __fdividef(act, 1.f + __expf(-act)) * lin * s_h * hm;
+                            const unsigned short hi = f32_to_f16_sat(val);
+                            if (store) {
+                                reinterpret_cast<unsigned short*>(A.h16)[(size_t)pos * R + r] = hi;
+                                if (wide) reinterpret_cast<unsigned short*>(A.h16lo)[(size_t)pos * R + r] =
+                                    f32_to_f16_sat((val - __half2float(__ushort_as_half(hi))) * pow2i(kLoShift));
+                            }
+                        }
                     }
                 }
-            return;
-        }
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int n = nt * 8 + tq * 2 + i;
-                if (n < ntok) {
-                    const float hs = A.hscale[pos0 + n];
-                    yp[(size_t)(pos0 + n) * C + row0 + mt * 16 + g] = sum[nt][i] * hs * so0;
-                    yp[(size_t)(pos0 + n) * C + row0 + mt * 16 + g + 8] = sum[nt][2 + i] * hs * so1;
-                }
             }
-        return;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(buf));
+            ++it;
+        }
+        }
     }
-
-    // S4 epilogue: thread holds U (sum[.][0..1]) and G (sum[.][2..3]) of row r for tokens 2tq, 2tq+1 of each n-tile.
-    // Per-pair power of two 2^f for the fp16 intermediate s_r h_r: |u|, |g| ~ s * 32 * |x| (codes have
-    // rms ~ 127/4) and |h| ~ u g / 2, so s h ~ s^3 * 512 |x|^2 for the row with the LARGEST scale of the expert
-    // (d.hexp = exponent of that s^3, from the routing kernel's statistics CTAs). That magnitude is placed at 2^-2:
-    // what matters to the down projection is the error relative to its largest terms, so the rows that carry the
-    // sum keep 11 bits with room for values 2^17 above the estimate, rows whose scale is much smaller may fall
-    // into fp16's subnormals (absolute error 2^-25 against terms near 2^-2), and nothing overflows (the store
-    // saturates).
-    const __nv_bfloat16* sc = reinterpret_cast<const __nv_bfloat16*>(blob + 3 * per);
-    const int r = row0 + mt * 8 + g;
-    // s_u, s_g: scales of the up and gate rows; s_h: what is folded into the intermediate for the down projection.
-    // Shared format: all three are s_r and s h ~ s^3; per-matrix: s1, s3 and 1, so h ~ s^2.
-    const float s_u = __bfloat162float(sc[r]);
-    const float s_g = A.per_matrix ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_gate)[r]) : s_u;
-    const float s_h = A.per_matrix ? 1.f : s_u;
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int n = nt * 8 + tq * 2 + i;
-            if (n < ntok) {
-                const int pos = pos0 + n;
-                const int tok = A.row_token[pos];
-                const int f = max(-120, min(120, -(d.hexp + 11 + 2 * expo(A.xnorm[tok]))));
-                if (row0 == 0 && mt == 0 && g == 0) A.hscale[pos] = pow2i(-f);
-                const float xs = A.xscale[tok];
-                const float u = sum[nt][i] * (xs * s_u), gt = sum[nt][2 + i] * (xs * s_g);
-                const float h = A.act_on_w1 ? silu(u) * gt : silu(gt) * u;
-                const float v = h * s_h * pow2i(f);
-                const unsigned short hi = f32_to_f16_sat(v);
-                reinterpret_cast<unsigned short*>(A.h16)[(size_t)pos * R + r] = hi;
-                if (d.wide)
-                    reinterpret_cast<unsigned short*>(A.h16lo)[(size_t)pos * R + r] =
-                        f32_to_f16_sat((v - __half2float(__ushort_as_half(hi))) * pow2i(kLoShift));
-            }
-        }
+    // ---------------------------------------------------- common exit
+    tc_fence_before();
+    __syncthreads();
+    if (s_abort) {                       // a wait ran out: give the copies in flight time to land (they take microseconds)
+        if (tid == 0) atomicOr(A.status, 2);
+        for (int i = 0; i < 50; ++i) __nanosleep(1000);
+    }
+    if (warp == 2) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
     }
 }
 
-template <bool DOWN, typename I, bool REHEARSE = false>
-__global__ void __launch_bounds__(kThreads, 2) k_ffn(FfnArgs A) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ ItemTable tab;
-    unsigned char* ringA = smem;
-    // The schedule comes from the routing kernel, which has completed once the up/gate kernel has started; the
-    // down kernel may therefore read it before its own wait (the up/gate kernel may not).
-    // The down kernel goes further before its wait: it also issues the weight copies of its first step, which depend
-    // on the routing alone, so the weight stream restarts while the up/gate kernel drains. Every CTA still waits
-    // before it exits or signals its dependents.
-    const int pair = threadIdx.x >> 6;
-    const int S = DOWN ? A.down_splits : 1;
-    const I n_mg = DOWN ? A.C / (16 * kMT) : A.R / (8 * kMT);
-    const I per_tb = n_mg * S;
-    const int w_full = block_cost(DOWN ? 1 : 0, 4);
-    I u = 0, u1 = 0;
-    const unsigned sA = (unsigned)__cvta_generic_to_shared(ringA);
+// ---------------------------------------------------------------------------------------------
+struct DigitArgs {
+    const __half* x16; const int32_t* row_token; const int32_t* count; const int32_t* offset; const int32_t* slot_map; const int32_t* hexp;
+    const float* xscale; const float* xnorm; const Sched* sched;
+    float* xs_pos; float* hm_pos; float* hscale; float* hs_pos;
+    const __half* h16; const __half* h16lo;
+    int8_t* planes; size_t plane;            // bytes between two planes
+    int n_all, cols;
+};
+__device__ __forceinline__ int expert_of(const DigitArgs& D, int pos, int* s_e) {
+    for (int e = threadIdx.x; e < D.n_all; e += blockDim.x)
+        if (D.offset[e] <= pos && pos < D.offset[e + 1]) *s_e = e;
+    __syncthreads();
+    return *s_e;
+}
 
-    // Describes the step that starts at unit v (valid = false past the end of this CTA's range). S5 of a wide-range
-    // expert carries two fp16 windows per token, so a block of more than 16 tokens is taken as two steps over the
-    // same units: half 0 = its first 16 tokens, half 1 = the rest.
-    auto decode = [&](I v, int half) {
-        StepDesc d;
-        d.valid = v < u1;
-        d.nstep = 0; d.nt = 0; d.active = false; d.blob = nullptr; d.hexp = 0; d.wide = false; d.last_half = true;
-        d.row0 = d.k0 = d.klen = d.split = d.pos0 = d.ntok = 0;
-        if (!d.valid) return d;
-        const int tbg = (int)(v / per_tb);
-        int lo = 0, hi = tab.n_active - 1;                  // largest a with tb_prefix[a] <= tbg
-        while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (tab.tb_prefix[mid] <= tbg) lo = mid; else hi = mid - 1; }
-        const int e = min((int)tab.act_expert[lo], A.n_all - 1);     // (the clamp only matters to the rehearsal pass)
-        const int tb = tbg - tab.tb_prefix[lo];
-        const int rem = (int)(v - (I)tbg * per_tb);            // < per_tb = row groups x slices
-        d.split = rem / (int)n_mg;
-        const int mg = rem - d.split * (int)n_mg;
-        const I left = u1 - v, in_group = n_mg - mg;
-        const I steps = (left + kPairs - 1) / kPairs;
-        d.nstep = (int)min(in_group, (left + steps - 1) / steps);
-        const int cnt = A.count[e];
-        d.pos0 = A.offset[e] + tb * kTokBlock;
-        d.ntok = min(kTokBlock, cnt - tb * kTokBlock);
-        d.nt = (d.ntok + 7) >> 3;
-        d.wide = A.hexp[kMaxExperts + e] != 0;
-        if (DOWN && d.wide) {
-            d.last_half = half == 1 || d.ntok <= kTokBlock / 2;
-            d.pos0 += half * (kTokBlock / 2);
-            d.ntok = min(kTokBlock / 2, d.ntok - half * (kTokBlock / 2));
-            d.nt = 2 * ((d.ntok + 7) >> 3);
-        }
-        d.blob = static_cast<const unsigned char*>(A.slots[max(A.slot_map[e], 0)]);     // (an active expert has a slot)
-        if (!DOWN) d.hexp = A.hexp[e];
-        d.k0 = DOWN ? d.split * A.down_slice : 0;
-        d.klen = DOWN ? min(A.down_slice, A.R - d.k0) : A.C;
-        d.row0 = (mg + pair) * (DOWN ? 16 * kMT : 8 * kMT);
-        d.active = pair < d.nstep;
-        return d;
+// Activation digits of one position (x16 is the row scaled by a power of two, largest value in [2^13, 2^14): times 2^8) and the
+// factors of its SwiGLU epilogue: 2^e, and the power of two 2^f that places the fp16 intermediate. |u|, |g| ~ s * 32 * |x| (codes
+// have rms ~ 127 / 4) and |h| ~ u g / 2, so s h ~ s^3 * 512 |x|^2 for the row with the LARGEST scale of the expert (hexp =
+// exponent of that s^3, from the routing kernel's statistics CTAs; per-matrix format: of s1 s3). That magnitude is placed at 2^-2.
+__global__ void __launch_bounds__(256) k_digits_x(DigitArgs D) {
+    __shared__ int s_e;
+    pdl_wait();
+    pdl_launch();
+    const int pos = blockIdx.x, e = expert_of(D, pos, &s_e);
+    if (D.count[e] >= D.sched->tc_min[0] || D.slot_map[e] < 0) return;       // the other kernel's, or not resident
+    const int tok = D.row_token[pos];
+    const uint4* src = reinterpret_cast<const uint4*>(D.x16 + (size_t)tok * D.cols);
+    uint2* dst = reinterpret_cast<uint2*>(D.planes + (size_t)pos * D.cols);
+    for (int i = threadIdx.x; i < D.cols / 8; i += 256) {
+        const uint4 v = src[i];
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+        const Digits8 d = digits_of_x16(w);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) dst[p * (D.plane / 8) + i] = d.p[p];
+    }
+    if (threadIdx.x == 0) {
+        const int f = max(-120, min(120, -(D.hexp[e] + 11 + 2 * expo(D.xnorm[tok]))));
+        D.xs_pos[pos] = D.xscale[tok] * (1.f / 256.f);
+        D.hm_pos[pos] = pow2i(f);
+        D.hscale[pos] = pow2i(-f);
+    }
+}
+
+// Digits of the intermediate of one position (of a wide-range expert: both fp16 windows together, 22 bits), scaled by the row's own largest value.
+// Launches its dependents at once: the down kernel may request its weights while the up/gate kernel drains (what it reads before
+// its own wait comes from the routing kernels, complete before the up/gate kernel started).
+constexpr int kDigitThreads = 1024, kDigitVecs = 2;       // most threads; a row of 16384 in one round of loads (longer rows take more rounds)
+__global__ void __launch_bounds__(kDigitThreads, 2) k_digits_h(DigitArgs D) {
+    __shared__ int s_e;
+    __shared__ float s_max[kDigitThreads / 32];
+    pdl_launch();
+    const int pos = blockIdx.x, e = expert_of(D, pos, &s_e);           // (routing results, see above)
+    const bool mine = D.count[e] < D.sched->tc_min[1] && D.slot_map[e] >= 0, wide = D.hexp[kMaxExperts + e] != 0;
+    pdl_wait();
+    if (!mine) return;
+    const uint4* hi = reinterpret_cast<const uint4*>(D.h16 + (size_t)pos * D.cols);
+    const uint4* lo = reinterpret_cast<const uint4*>(D.h16lo + (size_t)pos * D.cols);
+    const int n = D.cols / 8;
+    auto value = [&](const uint4& a, const uint4& b, int j) {
+        const unsigned wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
+        const float h = __half2float(__ushort_as_half((unsigned short)(wa[j >> 1] >> (16 * (j & 1)))));
+        return wide ? fmaf(__half2float(__ushort_as_half((unsigned short)(wb[j >> 1] >> (16 * (j & 1))))), pow2i(-kLoShift), h) : h;
     };
-
-    // Table, partition and the description of the first step. The up/gate kernel runs this twice: once as a rehearsal
-    // BEFORE its wait, on whatever the schedule memory holds (results discarded; every index it forms is clamped or
-    // stays inside the table), then for real. The CTAs sit in that wait for most of the routing kernel anyway, and the
-    // step streams more than the L2 holds, so each kernel's instructions come from DRAM again every step: the rehearsal
-    // takes those misses off the critical path (same loop body, so the same instruction addresses). Steps of up to 16
-    // tokens do it (fine-grained layer, 4 / 16 tokens: 0.0540 -> 0.0532 / 0.0703 -> 0.0690 ms per step); alone, without
-    // a predecessor to wait for, the kernel is 1.7 us slower for it, and from 32 tokens on the step gains nothing.
-    int half = 0;
-    StepDesc cur;
-    I total = 0;
-#pragma unroll 1
-    for (int pass = REHEARSE ? 0 : 1; pass < 2; ++pass) {
-        if (!DOWN && pass == 1) { if (REHEARSE) __syncthreads(); pdl_wait(); pdl_launch(); }
-        load_table(tab, A.sched, DOWN ? 1 : 0);
-        total = (I)tab.total_tb * per_tb;
-        const I cost = (I)tab.w_prefix[tab.n_active] * per_tb;
-        u = unit_at<I>(tab, cost * (I)blockIdx.x / (I)gridDim.x, per_tb, w_full);
-        u1 = unit_at<I>(tab, cost * (I)(blockIdx.x + 1) / (I)gridDim.x, per_tb, w_full);
-        cur = decode(u, 0);
-    }
-    if (total == 0 || !cur.valid) { if (DOWN) { pdl_wait(); pdl_launch(); } return; }
-    CopyState cs = DOWN ? start_step_weights<DOWN>(A, cur, sA) : start_step<DOWN>(A, cur, sA);
-    if (DOWN) {
-        pdl_wait();
-        pdl_launch();
-        start_step_acts(cs, cur);
-    }
-    while (cur.valid) {
-        if (cur.last_half) { u += cur.nstep; half = 0; } else half = 1;
-        const StepDesc next = decode(u, half);
-        CopyState cs_next = cs;
-        switch (cur.nt) {
-            case 1: ffn_step<DOWN, 1>(A, cur, cs, next, cs_next, ringA); break;
-            case 2: ffn_step<DOWN, 2>(A, cur, cs, next, cs_next, ringA); break;
-            case 3: ffn_step<DOWN, 3>(A, cur, cs, next, cs_next, ringA); break;
-            default: ffn_step<DOWN, 4>(A, cur, cs, next, cs_next, ringA); break;
+    uint4 a[kDigitVecs], b[kDigitVecs];
+    auto fetch = [&](int i0) {
+#pragma unroll
+        for (int q = 0; q < kDigitVecs; ++q) {
+            const int i = i0 + q * blockDim.x + threadIdx.x;
+            a[q] = i < n ? hi[i] : make_uint4(0, 0, 0, 0);
+            b[q] = wide && i < n ? lo[i] : make_uint4(0, 0, 0, 0);
         }
-        cur = next;
-        cs = cs_next;
+    };
+    const int round = kDigitVecs * blockDim.x;
+    float m = 0.f;
+    for (int i0 = (n - 1) / round * round; i0 >= 0; i0 -= round) {       // the first round last: it stays in registers
+        fetch(i0);
+#pragma unroll
+        for (int q = 0; q < kDigitVecs; ++q)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(value(a[q], b[q], j)));
     }
+    m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = __uint_as_float(__reduce_max_sync(0xffffffffu, (threadIdx.x & 31) < blockDim.x >> 5 ? __float_as_uint(s_max[threadIdx.x & 31]) : 0u));
+    const int ex = digit_exponent(m);
+    const float up = pow2i(21 - ex);
+    uint2* dst = reinterpret_cast<uint2*>(D.planes + (size_t)pos * D.cols);
+    for (int i0 = 0; i0 < n; i0 += round) {
+        if (i0 > 0) fetch(i0);
+#pragma unroll
+        for (int q = 0; q < kDigitVecs; ++q) {
+            const int i = i0 + q * blockDim.x + threadIdx.x;
+            if (i >= n) continue;
+            Digits8 d;
+            clear_digits(d);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) set_digits(d, j, __float2int_rn(value(a[q], b[q], j) * up));
+#pragma unroll
+            for (int p = 0; p < 3; ++p) dst[p * (D.plane / 8) + i] = d.p[p];
+        }
+    }
+    if (threadIdx.x == 0) D.hs_pos[pos] = pow2i(ex - 21) * D.hscale[pos];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -702,57 +664,121 @@ __global__ void __launch_bounds__(kCombineThreads) k_combine(CombineArgs A) {
     }
 }
 
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+bool encode_bytes(EncodeTiledFn fn, void* out, void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(reinterpret_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_UINT8, rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 FfnArgs make_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map) {
     FfnArgs A;
     A.slots = slots; A.slot_map = slot_map;
     A.sched = ws_ptr<Sched>(ctx, ctx->lay.sched);
     A.count = ws_ptr<int32_t>(ctx, ctx->lay.count);
     A.offset = ws_ptr<int32_t>(ctx, ctx->lay.offset);
-    A.row_token = ws_ptr<int32_t>(ctx, ctx->lay.row_token);
-    A.xscale = ws_ptr<float>(ctx, ctx->lay.xscale);
-    A.xnorm = ws_ptr<float>(ctx, ctx->lay.xnorm);
-    A.hscale = ws_ptr<float>(ctx, ctx->lay.hscale);
+    A.wmaps = ws_ptr<CUtensorMap>(ctx, ctx->lay.wmaps);
     A.hexp = ws_ptr<int32_t>(ctx, ctx->lay.hexp);
-    A.x16 = ws_ptr<__half>(ctx, ctx->lay.x16);
+    A.xs_pos = ws_ptr<float>(ctx, ctx->lay.xs_pos);
+    A.hm_pos = ws_ptr<float>(ctx, ctx->lay.hm_pos);
+    A.hs_pos = ws_ptr<float>(ctx, ctx->lay.hs_pos);
     A.h16 = ws_ptr<__half>(ctx, ctx->lay.h16);
     A.h16lo = ws_ptr<__half>(ctx, ctx->lay.h16lo);
     A.ypart = ws_ptr<float>(ctx, ctx->lay.ypart);
+    A.status = ws_ptr<int32_t>(ctx, ctx->lay.status);
     A.R = ctx->cfg.ffn; A.C = ctx->cfg.hidden; A.act_on_w1 = ctx->cfg.act_on_w1;
-    A.down_splits = ctx->down_splits; A.down_slice = ctx->down_slice;
     A.per_matrix = ctx->cfg.format == MIRA_FORMAT_PER_MATRIX;
-    A.n_all = ctx->cfg.n_experts + ctx->cfg.n_shared;
+    // An expert gets at most one position per token, so a small batch needs no wide activation tile and has a deeper ring.
+    A.tile_tok = std::min(kMaxTok, (ctx->route_T + 7) / 8 * 8);
+    A.n_all = Et(ctx->cfg);
+    A.b_box = ((3 * A.tile_tok + 15) / 16 * 16) * kKBox;           // (the MMA's columns are a multiple of 16)
+    // Two boxes per stage (one wait and one commit per eight MMAs) while at least four such stages fit.
+    A.boxes = 2 * (kABox + A.b_box) * 4 <= kRingBytes ? 2 : 1;
+    A.stage_bytes = A.boxes * (kABox + A.b_box);
+    A.stages = std::min(kMaxStages, kRingBytes / A.stage_bytes);
+    A.token_order = ctx->route_T <= kTokenOrderMax;
+    A.T = ctx->route_T;
+    A.row_token = ws_ptr<int32_t>(ctx, ctx->lay.row_token);
+    A.xscale = ws_ptr<float>(ctx, ctx->lay.xscale); A.xnorm = ws_ptr<float>(ctx, ctx->lay.xnorm);
+    A.hscale = ws_ptr<float>(ctx, ctx->lay.hscale);
+    A.splits = stream_down_splits(ctx);
     A.ypart_stride = (long)ctx->route_T * (ctx->route_k + ctx->cfg.n_shared) * ctx->cfg.hidden;
     return A;
 }
-
-// Whether every cost position of a step fits 31 bits: cost of all token blocks (at most 32 per block; a step has at
-// most pairs / 32 + experts blocks) x units per block x CTAs.
-bool fits_32(const mira_ctx* ctx, long long per_tb) {
-    const long long pairs = (long long)ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
-    const long long blocks = pairs / kTokBlock + ctx->cfg.n_experts + ctx->cfg.n_shared;
-    return blocks * 32 * per_tb * (2LL * ctx->n_sm + 1) < (1LL << 31);
+DigitArgs digit_args(mira_ctx* ctx, const int32_t* slot_map, size_t planes, int cols) {
+    DigitArgs D;
+    D.x16 = ws_ptr<__half>(ctx, ctx->lay.x16); D.row_token = ws_ptr<int32_t>(ctx, ctx->lay.row_token);
+    D.count = ws_ptr<int32_t>(ctx, ctx->lay.count); D.offset = ws_ptr<int32_t>(ctx, ctx->lay.offset);
+    D.slot_map = slot_map; D.hexp = ws_ptr<int32_t>(ctx, ctx->lay.hexp);
+    D.xscale = ws_ptr<float>(ctx, ctx->lay.xscale); D.xnorm = ws_ptr<float>(ctx, ctx->lay.xnorm); D.sched = ws_ptr<Sched>(ctx, ctx->lay.sched);
+    D.xs_pos = ws_ptr<float>(ctx, ctx->lay.xs_pos); D.hm_pos = ws_ptr<float>(ctx, ctx->lay.hm_pos);
+    D.hscale = ws_ptr<float>(ctx, ctx->lay.hscale); D.hs_pos = ws_ptr<float>(ctx, ctx->lay.hs_pos);
+    D.h16 = ws_ptr<__half>(ctx, ctx->lay.h16); D.h16lo = ws_ptr<__half>(ctx, ctx->lay.h16lo);
+    D.planes = ws_ptr<int8_t>(ctx, planes);
+    D.plane = (size_t)Pmax(ctx->cfg) * cols;
+    D.n_all = Et(ctx->cfg); D.cols = cols;
+    return D;
+}
+template <bool DOWN> cudaError_t launch_ffn(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, cudaStream_t st) {
+    static_assert(sizeof(DigitMaps) == sizeof(ctx->tmap_digits[0]), "tensor map storage");
+    DigitMaps maps;
+    memcpy(&maps, ctx->tmap_digits[DOWN ? 1 : 0], sizeof(maps));
+    return launch_pdl(k_ffn<DOWN>, dim3(ctx->n_sm), dim3(kThreads), (size_t)kRingBytes + 1024, st, make_args(ctx, slots, slot_map), maps);
 }
 
 }  // namespace
 
+// The down projection has only hidden / 32 units per expert, so its reduction is cut into slices (their sums meet in S6): without
+// them 8 experts of 4096 hidden rows are 1.7 items per CTA (128 tokens: 144 us without, 107 with slices).
+int stream_down_splits(const mira_ctx* ctx) { return ctx->down_splits; }
+
+// Tensor maps of the digit planes (the caller's workspace, whose address is fixed at mira_create) and the templates of the weight
+// maps: expert e's copies (workspace, wmaps) get the address of its blob from the routing kernels, see make_weight_maps.
+bool build_stream_maps(mira_ctx* ctx) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess || p == nullptr || q != cudaDriverEntryPointSuccess)
+        return false;
+    const EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(p);
+    const cuuint64_t P = Pmax(ctx->cfg), C = ctx->cfg.hidden, R = ctx->cfg.ffn;
+    for (int i = 0; i < kDigitMaps; ++i)
+        for (int d = 0; d < 2; ++d) {
+            const cuuint64_t cols = d ? R : C, dims[3] = {cols, P, 3}, str[2] = {cols, cols * P};
+            const cuuint32_t box[3] = {kKBox, (cuuint32_t)(8 * (i + 1)), 3};
+            if (!encode_bytes(fn, ctx->tmap_digits[d][i], ctx->ws + (d ? ctx->lay.hq : ctx->lay.xq), 3, dims, str, box)) return false;
+        }
+    unsigned char tmpl[kWeightMaps][128];
+    const cuuint64_t up_dims[3] = {C, 2, R}, up_str[2] = {2 * R * C, C};           // W1^ and W3^ rows in turn
+    const cuuint64_t dn_dims[2] = {R, C}, dn_str[1] = {R};
+    for (cuuint32_t i = 0; i < 4; ++i) {
+        const cuuint32_t up_box[3] = {kKBox, 2, 16 * (i + 1)}, dn_box[2] = {kKBox, 32 * (i + 1)};
+        if (!encode_bytes(fn, tmpl[i], ctx->ws, 3, up_dims, up_str, up_box) || !encode_bytes(fn, tmpl[4 + i], ctx->ws, 2, dn_dims, dn_str, dn_box)) return false;
+    }
+    return cudaMemcpy(ctx->ws + ctx->lay.wmaps + (size_t)kMaxExperts * kWeightMaps * 128, tmpl, sizeof(tmpl), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+
 mira_status launch_up_gate(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, cudaStream_t st) {
-    FfnArgs A = make_args(ctx, slots, slot_map);
     ProfScope ps(ctx, MIRA_K_UP_GATE, st);
-    if (ctx->route_T <= 16 && fits_32(ctx, ctx->cfg.ffn / (8 * kMT)))        // small steps rehearse their start-up code, see k_ffn
-        MIRA_CUDA_OK(launch_pdl(k_ffn<false, int, true>, dim3(ctx->n_sm * 2), dim3(kThreads), kSmemBytes, st, A));
-    else if (fits_32(ctx, ctx->cfg.ffn / (8 * kMT))) MIRA_CUDA_OK(launch_pdl(k_ffn<false, int>, dim3(ctx->n_sm * 2), dim3(kThreads), kSmemBytes, st, A));
-    else MIRA_CUDA_OK(launch_pdl(k_ffn<false, long long>, dim3(ctx->n_sm * 2), dim3(kThreads), kSmemBytes, st, A));
+    if (ctx->route_T > kTokenOrderMax) {          // else the routing kernel has written the digits
+        const int P = ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
+        MIRA_CUDA_OK(launch_pdl(k_digits_x, dim3(P), dim3(256), 0, st, digit_args(ctx, slot_map, ctx->lay.xq, ctx->cfg.hidden)));
+        ctx->launches += 1;
+    }
+    MIRA_CUDA_OK(launch_ffn<false>(ctx, slots, slot_map, st));
     ctx->launches += 1;
     MIRA_CUDA_OK(cudaGetLastError());
     return MIRA_OK;
 }
 
 mira_status launch_down(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, cudaStream_t st) {
-    FfnArgs A = make_args(ctx, slots, slot_map);
     ProfScope ps(ctx, MIRA_K_DOWN, st);
-    if (fits_32(ctx, (long long)(ctx->cfg.hidden / (16 * kMT)) * ctx->down_splits)) MIRA_CUDA_OK(launch_pdl(k_ffn<true, int>, dim3(ctx->n_sm * 2), dim3(kThreads), kSmemBytes, st, A));
-    else MIRA_CUDA_OK(launch_pdl(k_ffn<true, long long>, dim3(ctx->n_sm * 2), dim3(kThreads), kSmemBytes, st, A));
-    ctx->launches += 1;
+    const int P = ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
+    const int threads = std::min(kDigitThreads, (ctx->cfg.ffn / 8 + 32 * kDigitVecs - 1) / (32 * kDigitVecs) * 32);
+    MIRA_CUDA_OK(launch_pdl(k_digits_h, dim3(P), dim3(threads), 0, st, digit_args(ctx, slot_map, ctx->lay.hq, ctx->cfg.ffn)));
+    MIRA_CUDA_OK(launch_ffn<true>(ctx, slots, slot_map, st));
+    ctx->launches += 2;
     MIRA_CUDA_OK(cudaGetLastError());
     return MIRA_OK;
 }
@@ -778,11 +804,8 @@ mira_status launch_combine(mira_ctx* ctx, int T, int k, int splits, int tc_split
 }
 
 mira_status set_ffn_attributes() {
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBytes)));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false, int, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBytes)));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBytes)));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false, long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBytes)));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true, long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBytes)));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
     return MIRA_OK;
 }
 

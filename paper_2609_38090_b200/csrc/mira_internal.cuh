@@ -12,9 +12,11 @@ namespace mira {
 
 constexpr int kMaxExperts = 256;   // E + n_shared
 constexpr int kMaxTopK = 16;
-constexpr int kTokBlock = 32;      // tokens of one expert handled by one work item (4 MMA n-tiles)
-constexpr int kChunk = 64;         // reduction-dimension bytes of one weight row per pipeline stage
-constexpr int kDownSlice = 4096;   // nominal reduction length of one split of the down projection
+constexpr int kDownSlice = 4096;   // nominal reduction length of one slice of the down projection
+constexpr int kWeightMaps = 8;     // tensor maps per expert: up/gate tiles of 32, 64, 96, 128 MMA rows, then down tiles
+constexpr int kTokenOrderMax = 16; // up to here the routing kernels write the activations' digit planes in token order and every expert's
+                                   // up/gate tile holds all tokens of the batch (its columns beyond the expert's own are not read)
+constexpr int kDigitMaps = 10;     // tensor maps of a digit-plane matrix: boxes of 8, 16, ..., 80 positions
 // The fp16 intermediate v = s_r h_r 2^f of a wide-range expert is kept as two fp16 values, hi = fp16(v) and
 // lo = fp16((v - hi) * 2^kLoShift), both saturating: together they hold 11 bits or more of every |v| in
 // [2^-38, 2^16). The down projection multiplies both by the same weight fragments and adds the second sum scaled
@@ -23,27 +25,15 @@ constexpr int kLoShift = 24;
 
 // Device-resident schedule written by the grouping kernel and read by the expert kernels.
 struct Sched {
-    int32_t n_active;                  // experts with at least one pair AND a resident slot
+    int32_t n_active;                  // experts with at least one pair AND a resident slot (and in the wave)
     int32_t act_expert[kMaxExperts];   // active expert ids, ascending
+    uint32_t act_mask[kMaxExperts / 32];     // the same set as bits
     // A step may split its experts between the two kernel families ("hybrid" step): an active expert with fewer than
     // tc_min[p] pairs is taken by the weight-streaming kernel of projection p (0 up/gate, 1 down), the others by
-    // the tcgen05 kernel (tc_min = 0: all tensor-core; INT_MAX: all streaming). The streaming kernels' work lists:
+    // the tcgen05 kernel (tc_min = 0: all tensor-core; INT_MAX: all streaming).
     int32_t tc_min[2];
-    int32_t total_tb[2];               // token blocks of the streaming kernel of projection p
-    int32_t tb_prefix[2][kMaxExperts + 1];   // exclusive prefix sum of those token blocks per active expert (0 blocks for
-                                             // an expert the tensor-core kernel takes)
-    // Exclusive prefix sums of the COST of the token blocks, [0] for the up/gate kernel, [1] for the down kernel.
-    // A block of 1-8, 9-16, 17-24, 25-32 tokens costs block_cost(., 1..4): the streaming kernels split the work
-    // between CTAs by cost, not by block count. Alone, a full block takes about 1.5x the time of an 8-token block
-    // (uniform counts: 171 / 193 / 218 / 258 us up/gate, 89 / 97 / 117 / 137 us down); in a batch with mixed counts
-    // the gap is wider, because the CTAs of small blocks speed up while the others are compute bound and leave
-    // them memory bandwidth, so the costs are those that balanced skewed 16- and 32-token batches best.
-    int32_t w_prefix[2][kMaxExperts + 1];
+    uint32_t ticket[2];                // items of the streaming kernel of projection p that its CTAs have drawn
 };
-__host__ __device__ constexpr int block_cost(int which, int n_tiles) {       // which: 0 up/gate, 1 down; n_tiles 1..4
-    return which == 0 ? (n_tiles <= 1 ? 16 : n_tiles == 2 ? 22 : n_tiles == 3 ? 27 : 31)
-                      : (n_tiles <= 1 ? 16 : n_tiles == 2 ? 22 : n_tiles == 3 ? 27 : 32);
-}
 
 // Where the scale vectors of a compressed expert live (byte offsets from the start of the blob) and how they
 // enter the FFN, for the two formats. Shared scale: one vector s[R] scales the up and gate rows and is folded
@@ -87,6 +77,10 @@ struct Layout {
     size_t hm_pos;      // float [Pmax]    per position: 2^f applied to the fp16 intermediate (tensor-core path)
     size_t sum_pos;     // float [Pmax]    per position: sum of the token's fp16 activations (tensor-core path)
     size_t h16;         // half  [Pmax][R]
+    size_t xq;          // int8 [3][Pmax][C] digit planes of the activations in position order (weight-streaming kernels)
+    size_t hq;          // int8 [3][Pmax][R] digit planes of the intermediate
+    size_t hs_pos;      // float [Pmax] per position: undo factor of the intermediate's digits and placement
+    size_t wmaps;       // 128-byte tensor maps [kMaxExperts][kWeightMaps] of the resident experts, then their templates
     size_t ypart;       // float [S][Pmax][C] split partial sums of the down projection
     size_t pred;        // float [head_chunks][C + E] token sums of the linear head's batches ...
     size_t mix;         // ... and of the MixtureHead's
@@ -110,6 +104,7 @@ struct mira_ctx {
     alignas(64) unsigned char tmap_h16[6][128];    // CUtensorMaps of h16, likewise
     alignas(64) unsigned char tmap_h16lo[6][128];  // CUtensorMaps of h16lo, likewise
     alignas(64) unsigned char tmap_half[3][6][128]; // x16p, h16, h16lo with boxes of 16, 32, ..., 96 rows (two-SM kernels)
+    alignas(64) unsigned char tmap_digits[2][mira::kDigitMaps][128];   // digit planes of the activations, of the intermediate
     bool tensor_path_ok = false;
     bool force_decode_path = false;
     int tc_layout = 0;                 // 0: chosen per step; 1..3 force a tile layout of the tensor-core kernels (MIRA_OPT_TENSOR_LAYOUT)
@@ -128,7 +123,6 @@ struct mira_ctx {
     int device;
     int n_sm;
     int down_splits;        // S
-    int down_slice;         // reduction length per split (multiple of 64)
     int route_T;            // T of the last routing call (-1: none)
     int route_k;
     int64_t launches;
@@ -168,6 +162,8 @@ mira_status launch_pool(mira_ctx*, const float* token_scores, int T, int E, floa
 // expert_ffn.cu
 mira_status launch_up_gate(mira_ctx*, void* const* slots, const int32_t* slot_map, cudaStream_t);
 mira_status launch_down(mira_ctx*, void* const* slots, const int32_t* slot_map, cudaStream_t);
+bool build_stream_maps(mira_ctx*);
+int stream_down_splits(const mira_ctx*);     // reduction slices of the weight-streaming down kernel for the step last routed
 mira_status launch_combine(mira_ctx*, int T, int k, int splits, int tc_splits, int down_tc_min, void* out, cudaStream_t);
 int down_tc_slices(const mira_ctx*);     // reduction slices the tensor-core down kernel uses for the step last routed
 // expert_ffn_tc.cu (tcgen05 path for prefill-sized batches)
@@ -176,15 +172,21 @@ bool build_tensor_maps(mira_ctx*);
 mira_status launch_up_gate_tc(mira_ctx*, void* const* slots, const int32_t* slot_map, cudaStream_t);
 mira_status launch_down_tc(mira_ctx*, void* const* slots, const int32_t* slot_map, cudaStream_t);
 mira_status set_tc_attributes();
-// From how many tokens a step takes the tcgen05 kernel instead of the weight-streaming one, separately for the up/gate
-// and the down projection (measured, us per kernel, streaming / tcgen05: Mixtral shape up/gate 40 tokens 182 / 200,
-// 56 tokens 202 / 203, down 32 tokens 103 / 102, 40 tokens 115 / 104, 48 tokens 118 / 104; fine-grained shape with
-// 64 experts up/gate 16 tokens 38 / 42, 32 tokens 48 / 44, down 16 tokens 26 / 23, 32 tokens 30 / 27; below these
-// sizes the streaming kernels win: Mixtral shape 16 tokens 0.231 / 0.240 ms per step, fine-grained 4 tokens 0.055 /
-// 0.057). The down projection switches earlier: its exact conversion costs the streaming kernel more per weight.
-constexpr int kTensorPathMinTokens = 16;    // below, no buffers of the tensor path are laid out
-inline int tc_min_tokens_up(const mira_config& c) { return c.n_experts + c.n_shared > 16 ? 20 : 56; }
-inline int tc_min_tokens_down(const mira_config& c) { return c.n_experts + c.n_shared > 16 ? 16 : 40; }
+// Up to how many pairs per routed expert on average (T k / E) a step takes the weight-streaming kernel (int8 digits: bound by HBM,
+// but three MMA columns per token, 80 tokens per tile and a digit kernel before the down projection), beyond it the fp16
+// kernel (conversion in registers, 128 or 192 tokens per tile). Measured, us per step or kernel, streaming / fp16, at an
+// average of a pairs: up/gate, 8x7B shape (117 MB of up and gate codes per expert) a = 50: 212 / 252, 100: 303 / 336, 128:
+// 359 / 382; 8x22B a = 64: 428 / 436, 128: 708 / 677; hidden 2304, ffn 2816 (13 MB) a = 37: 197 / 230, 75: 284 / 295; hidden 4096,
+// ffn 1024 (8.4 MB) a = 21: 168 / 205, 58: 277 / 268; fine-grained (5.8 MB) a = 12: 74 / 77, 17: 87 / 81; hidden 1408, ffn 768
+// (2.2 MB) a = 21: 59 / 42: small experts pay for their tiles' ends. Down (with the digit kernel): hidden 4096 a = 50: 134 / 126, 21:
+// 110 / 123; hidden 2304 a = 17: 95 / 100, 37: 145 / 118; fine-grained (2048) a = 4: 38 / 35 (step 84 / 92), 8: 48 / 41 (equal
+// steps); hidden 1024 a = 19: 51 / 42: the digits of a pair are shared by the model-hidden rows.
+constexpr int kTensorPathMinTokens = 16;    // below, no buffers of the fp16 tensor path are laid out
+inline double stream_max_pairs(const mira_config& c, int projection) {
+    const double x = projection == 0 ? 8.0 * (2e-6 * c.hidden * c.ffn - 4.0) : (c.hidden - 1500) / 40.0;
+    const double least = projection == 0 ? 4.0 : 3.0, most = projection == 0 ? 110.0 : 60.0;
+    return x < least ? least : x > most ? most : x;
+}
 // Per projection (0 up/gate, 1 down): the pair count from which an expert of a T-token step goes to the tcgen05
 // kernel (0: every expert; INT_MAX: none). The same rule for every wave of a routed batch.
 void step_tc_min(const mira_ctx* ctx, int T, int k, int out_min[2]);
@@ -245,6 +247,32 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+// Digit planes. d0 2^16 + d1 2^8 + d2 = v, |v| < 2^22, digits in [-128, 127].
+__device__ __forceinline__ void digits(int v, int& d0, int& d1, int& d2) {
+    d2 = (int)(signed char)v;
+    v = (v - d2) >> 8;
+    d1 = (int)(signed char)v;
+    d0 = (v - d1) >> 8;
+}
+struct Digits8 { uint2 p[3]; };                  // eight consecutive values in three planes
+__device__ __forceinline__ void set_digits(Digits8& o, int j, int v) {       // j = 0, 1, ..., 7 in order, o zeroed before
+    int d0, d1, d2;
+    digits(v, d0, d1, d2);
+    const int s = 8 * (j & 3);
+    unsigned &a = j < 4 ? o.p[0].x : o.p[0].y, &b = j < 4 ? o.p[1].x : o.p[1].y, &c = j < 4 ? o.p[2].x : o.p[2].y;
+    a |= (unsigned)(d0 & 0xff) << s; b |= (unsigned)(d1 & 0xff) << s; c |= (unsigned)(d2 & 0xff) << s;
+}
+__device__ __forceinline__ void clear_digits(Digits8& o) { o.p[0] = o.p[1] = o.p[2] = make_uint2(0, 0); }
+// Digits of eight activations: fp16 values scaled so that the row's largest lies in [2^13, 2^14), times 2^8.
+__device__ __forceinline__ Digits8 digits_of_x16(const unsigned (&h2)[4]) {
+    Digits8 o;
+    clear_digits(o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        set_digits(o, j, __float2int_rn(__half2float(__ushort_as_half((unsigned short)(h2[j >> 1] >> (16 * (j & 1))))) * 256.f));
+    return o;
+}
 
 // Top-k by a warp.
 // The selection runs on 32-bit keys that order like the logits (sign-magnitude floats mapped to unsigned; -0 counts as

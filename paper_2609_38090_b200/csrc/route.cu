@@ -385,6 +385,7 @@ struct SchedArgs {
     // hexp[e]: exponent of the largest magnitude the intermediate of expert e is expected to reach per unit of |x|^2
     // (from the largest row scale of the blob in its slot), then the wide-range flags; written by the statistics CTAs.
     void* const* slots; int32_t* hexp;
+    unsigned char* wmaps;               // tensor maps of the experts' weights, then their templates (see make_weight_maps)
     int tc_min[2];                      // hybrid thresholds of the step (see Sched)
     int T, R, C, per_matrix, n_main;    // n_main: CTAs of the launch that are not statistics CTAs
 };
@@ -401,12 +402,29 @@ __device__ __forceinline__ float min8_bf16(const uint4& v) {
                  fminf(fminf(bf16lo(v.z), bf16hi(v.z)), fminf(bf16lo(v.w), bf16hi(v.w))));
 }
 
+// Tensor maps of expert e: copies of the templates (blobs have one shape) with the address of the blob in its slot. The slots
+// are known to the device only. Warp w < kWeightMaps makes map w: first W1^ and W3^ rows in turn, then W2^.
+__device__ __forceinline__ void make_weight_maps(const SchedArgs& S, int e, const unsigned char* blob) {
+    __shared__ __align__(128) unsigned s_map[kWeightMaps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp >= kWeightMaps) return;
+    s_map[warp][lane] = reinterpret_cast<const unsigned*>(S.wmaps + ((size_t)kMaxExperts * kWeightMaps + warp) * 128)[lane];
+    __syncwarp();
+    const unsigned sm = (unsigned)__cvta_generic_to_shared(s_map[warp]);
+    if (lane == 0)
+        asm volatile("tensormap.replace.tile.global_address.shared::cta.b1024.b64 [%0], %1;\n" ::"r"(sm), "l"(blob + (warp < kWeightMaps / 2 ? 0 : (size_t)S.R * S.C)) : "memory");
+    __syncwarp();
+    asm volatile("tensormap.cp_fenceproxy.global.shared::cta.tensormap::generic.release.gpu.sync.aligned [%0], [%1], 128;\n"
+                 ::"l"(S.wmaps + ((size_t)e * kWeightMaps + warp) * 128), "r"(sm) : "memory");
+}
+
 __device__ __forceinline__ void expert_stats(const SchedArgs& S, int e) {
     __shared__ float s_m[4][32];
     const bool sel = (S.mask.w[e >> 5] >> (e & 31)) & 1u;
     const int slot = (S.slots != nullptr && S.slot_map != nullptr && sel) ? S.slot_map[e] : -1;
     if (slot < 0) return;
     const unsigned char* blob = static_cast<const unsigned char*>(S.slots[slot]);
+    make_weight_maps(S, e, blob);
     const BlobFmt f = blob_fmt(S.per_matrix ? MIRA_FORMAT_PER_MATRIX : MIRA_FORMAT_SHARED, S.R, S.C);
     const uint4* su = reinterpret_cast<const uint4*>(blob + f.s_up);
     const uint4* sg = reinterpret_cast<const uint4*>(blob + f.s_gate);
@@ -441,125 +459,48 @@ __device__ __forceinline__ void expert_stats(const SchedArgs& S, int e) {
     }
 }
 
-// Serial tail of the schedule (one thread): the active experts in ascending order with the prefix sums of their
-// token blocks and of the blocks' costs. tb[i] = token blocks of expert i if it is active, else 0.
-__device__ __forceinline__ void write_schedule(Sched* sched, const int* tb, const int* count, int Etot,
-                                               int min_up, int min_down) {
-    int n = 0, au = 0, ad = 0, wu = 0, wd = 0;
-    sched->tc_min[0] = min_up; sched->tc_min[1] = min_down;
-    for (int i = 0; i < Etot; ++i) {
-        const int b = tb[i];
-        if (b > 0) {
-            sched->act_expert[n] = i;
-            sched->tb_prefix[0][n] = au; sched->tb_prefix[1][n] = ad;
-            sched->w_prefix[0][n] = wu; sched->w_prefix[1][n] = wd;
-            const int last = (count[i] - (b - 1) * kTokBlock + 7) >> 3;          // n-tiles of the last block, 1..4
-            if (count[i] < min_up) { wu += (b - 1) * block_cost(0, 4) + block_cost(0, last); au += b; }      // streaming up/gate
-            if (count[i] < min_down) { wd += (b - 1) * block_cost(1, 4) + block_cost(1, last); ad += b; }    // streaming down
-            ++n;
-        }
-    }
-    sched->tb_prefix[0][n] = au; sched->tb_prefix[1][n] = ad;
-    sched->w_prefix[0][n] = wu; sched->w_prefix[1][n] = wd;
-    sched->n_active = n;
-    sched->total_tb[0] = au; sched->total_tb[1] = ad;
-}
-
-// The same schedule written by kMaxExperts threads (thread e = expert e; b = its token blocks, 0 if it does not run):
-// five exclusive prefix sums over the experts (rank among the active ones, token blocks and costs of the two streaming
-// kernels), then every active expert writes its own entries. One loop body serves the five sums (the values wait in
-// shared memory), because this code runs once per step and is fetched cold: with 64 experts the serial loop took 3.7
-// us at the very end of the routing kernel, on the critical path of the step.
-// s_tmp: kSchedScratch ints; the calling threads (exactly kMaxExperts) meet at named barrier 1.
-constexpr int kSerialScheduleMax = 16;
-constexpr int kSchedScratch = 5 * kMaxExperts + 5 * (kMaxExperts / 32);
-__device__ __forceinline__ void write_schedule_parallel(Sched* sched, int b, int cnt, int min_up, int min_down, int* s_tmp) {
-    const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
-    constexpr int kW = kMaxExperts / 32;
-    int* s_v = s_tmp;                        // [5][kMaxExperts]: values, then their exclusive prefixes
-    int* s_w = s_tmp + 5 * kMaxExperts;      // [5][kW]: totals of the warps
-    {
-        const int last = b > 0 ? (cnt - (b - 1) * kTokBlock + 7) >> 3 : 1;            // n-tiles of the last block, 1..4
-        const bool up = b > 0 && cnt < min_up, dn = b > 0 && cnt < min_down;          // taken by the streaming kernel of that projection
-        s_v[e] = b > 0 ? 1 : 0;
-        s_v[kMaxExperts + e] = up ? b : 0;
-        s_v[2 * kMaxExperts + e] = dn ? b : 0;
-        s_v[3 * kMaxExperts + e] = up ? (b - 1) * block_cost(0, 4) + block_cost(0, last) : 0;
-        s_v[4 * kMaxExperts + e] = dn ? (b - 1) * block_cost(1, 4) + block_cost(1, last) : 0;
-    }
-#pragma unroll 1
-    for (int q = 0; q < 5; ++q) {
-        const int x = s_v[q * kMaxExperts + e];
-        int incl = x;
+// The schedule, from the mask words of the experts that run (every thread of the CTA calls it, at least kMaxExperts of them;
+// s_word holds the words): thread e writes expert e's place in the ascending list.
+__device__ __forceinline__ void write_schedule(const SchedArgs& S, const unsigned* s_word) {
+    const int e = threadIdx.x, w = e >> 5;
+    if (e < kMaxExperts && (s_word[w] >> (e & 31) & 1u)) {
+        int n = __popc(s_word[w] & ((1u << (e & 31)) - 1u));
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
-        if (lane == 31) s_w[q * kW + warp] = incl;
-        s_v[q * kMaxExperts + e] = incl - x;          // exclusive within the warp
+        for (int i = 0; i < kMaxExperts / 32; ++i) n += i < w ? __popc(s_word[i]) : 0;
+        S.sched->act_expert[n] = e;
     }
-    asm volatile("bar.sync 1, %0;\n" ::"n"(kMaxExperts) : "memory");
-    int before[5];
+    if (e < kMaxExperts / 32) S.sched->act_mask[e] = s_word[e];
+    if (e == 0) {
+        int n = 0;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) before[q] = 0;
-#pragma unroll 1
-    for (int w = 0; w < warp; ++w) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) before[q] += s_w[q * kW + w];
-    }
-    if (e == 0) { sched->tc_min[0] = min_up; sched->tc_min[1] = min_down; }
-    if (b > 0 || e == kMaxExperts - 1) {
-        // the last thread also writes the closing entry (its own exclusive prefix + its own value = the totals)
-        const int n = s_v[e] + before[0];
-        const int au = s_v[kMaxExperts + e] + before[1], ad = s_v[2 * kMaxExperts + e] + before[2];
-        const int wu = s_v[3 * kMaxExperts + e] + before[3], wd = s_v[4 * kMaxExperts + e] + before[4];
-        if (b > 0) {
-            sched->act_expert[n] = e;
-            sched->tb_prefix[0][n] = au; sched->tb_prefix[1][n] = ad;
-            sched->w_prefix[0][n] = wu; sched->w_prefix[1][n] = wd;
-        }
-        if (e == kMaxExperts - 1) {
-            // totals = this thread's exclusive prefixes plus its own values (recomputed: cheap, and only here)
-            const int last = b > 0 ? (cnt - (b - 1) * kTokBlock + 7) >> 3 : 1;
-            const bool up = b > 0 && cnt < min_up, dn = b > 0 && cnt < min_down;
-            const int nt = n + (b > 0 ? 1 : 0), tu = au + (up ? b : 0), td = ad + (dn ? b : 0);
-            const int cu = wu + (up ? (b - 1) * block_cost(0, 4) + block_cost(0, last) : 0);
-            const int cd = wd + (dn ? (b - 1) * block_cost(1, 4) + block_cost(1, last) : 0);
-            sched->tb_prefix[0][nt] = tu; sched->tb_prefix[1][nt] = td;
-            sched->w_prefix[0][nt] = cu; sched->w_prefix[1][nt] = cd;
-            sched->n_active = nt;
-            sched->total_tb[0] = tu; sched->total_tb[1] = td;
-        }
+        for (int i = 0; i < kMaxExperts / 32; ++i) n += __popc(s_word[i]);
+        S.sched->n_active = n;
+        S.sched->tc_min[0] = S.tc_min[0]; S.sched->tc_min[1] = S.tc_min[1];
+        S.sched->ticket[0] = S.sched->ticket[1] = 0u;
     }
 }
 
 // Called by every thread of a CTA of at least kMaxExperts threads. Thread e looks at expert e; a warp covers one word
 // of the masks, so the experts that run and the misses are collected with a ballot and cost one atomic per word
 // (not one per expert on the same word).
-__device__ __forceinline__ void schedule_body(const SchedArgs& S, const int* count, int Etot, int* s_tb, int* s_act) {
+__device__ __forceinline__ void schedule_body(const SchedArgs& S, const int* count, int Etot, int* s_tmp) {
     const int e = threadIdx.x;
+    unsigned* s_word = reinterpret_cast<unsigned*>(s_tmp);
     if (e < kMaxExperts) {
-        int tb = 0, act = 0, miss = 0;
-        if (e < Etot) {
-            const int c = count[e];
-            const bool sel = (S.mask.w[e >> 5] >> (e & 31)) & 1u;
-            if (c > 0 && sel) {
-                if (S.slot_map[e] >= 0) { act = 1; tb = (c + kTokBlock - 1) / kTokBlock; }
-                else miss = 1;
-            }
+        int act = 0, miss = 0;
+        if (e < Etot && count[e] > 0 && (S.mask.w[e >> 5] >> (e & 31) & 1u)) {
+            if (S.slot_map[e] >= 0) act = 1;
+            else miss = 1;
         }
-        s_tb[e] = tb; s_act[e] = act;
         const unsigned done_w = __ballot_sync(0xffffffffu, act), miss_w = __ballot_sync(0xffffffffu, miss);
         if ((e & 31) == 0) {
+            s_word[e >> 5] = done_w;
             if (done_w) atomicOr(S.done_mask + (e >> 5), done_w);
             if (miss_w && !S.quiet) { atomicOr(S.miss_mask + (e >> 5), miss_w); atomicOr(S.status, 1); }
         }
     }
     __syncthreads();
-    if (Etot <= kSerialScheduleMax) {        // few experts: one thread is as fast as the scans (8 experts: 0.5 us)
-        if (threadIdx.x == 0) write_schedule(S.sched, s_tb, count, Etot, S.tc_min[0], S.tc_min[1]);    // s_tb is 0 for inactive experts
-        return;
-    }
-    if (threadIdx.x >= kMaxExperts) return;
-    write_schedule_parallel(S.sched, s_tb[e], e < Etot ? count[e] : 0, S.tc_min[0], S.tc_min[1], s_act);
+    write_schedule(S, s_word);
 }
 
 // S3 for large batches, one CTA; with do_sched also the work schedule of a call that runs every routed expert.
@@ -573,28 +514,26 @@ __global__ void __launch_bounds__(1024) k_group(GroupArgs G, SchedArgs S, int do
     group_body<false>(G, s_count, s_off, s_hist);
     if (do_sched) {
         __syncthreads();
-        schedule_body(S, s_count, G.E + G.ns, s_off, s_hist);      // s_off and s_hist are free now
+        schedule_body(S, s_count, G.E + G.ns, s_off);      // s_off is free now
     }
 }
 
 __global__ void __launch_bounds__(256) k_schedule(const int32_t* __restrict__ count, int Etot, SchedArgs S) {
-    __shared__ int s_tb[kMaxExperts];
-    __shared__ int s_act[kSchedScratch];
+    __shared__ int s_word[kMaxExperts / 32];
     pdl_wait();            // the kernels of the wave before still read the schedule this one rewrites
     pdl_launch();
     if ((int)blockIdx.x >= S.n_main) { expert_stats(S, blockIdx.x - S.n_main); return; }
-    schedule_body(S, count, Etot, s_tb, s_act);
+    schedule_body(S, count, Etot, s_word);
 }
 
 // Fused S1-S3 for small batches: one CTA per token does the scores, the fp16 copy and the top-k; the
 // last CTA to finish (atomic ticket, no waiting) does the grouping and, if asked, the schedule.
 // Dynamic shared memory of k_route_token: the token row (2 C bytes), reused by the last CTA for the per-warp
-// histograms of the grouping step and as scratch of the schedule.
+// histograms of the grouping step.
 constexpr int kTokenSmemBytes = 4096;
 inline size_t token_smem(int C, int n_warps, int E) {
     size_t need = (size_t)C * 2;                                                  // the token row
     need = std::max(need, (size_t)n_warps * (size_t)E * 4);                       // the grouping CTA's histograms
-    need = std::max(need, (size_t)kSchedScratch * 4);                             // the schedule's scratch
     return std::max(need, (size_t)kTokenSmemBytes);
 }
 
@@ -602,6 +541,7 @@ struct TokenArgs {
     const __nv_bfloat16* x; int T, C; const __nv_bfloat16* W; const float* bias; int E;
     float* scores; __half* x16; float* xscale; float* xnorm; float* xsum; int k; int32_t* idx; float* wts;
     unsigned* ticket; int do_sched;
+    int8_t* xq; size_t xq_plane;        // digit planes in token order (NULL: not wanted), bytes between two planes
 };
 
 template <bool FEW, int THREADS>
@@ -659,6 +599,11 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
             o4[j] = *reinterpret_cast<const unsigned*>(&h);
         }
         og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+        if (A.xq != nullptr) {
+            const Digits8 d = digits_of_x16(o4);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A.xq + p * A.xq_plane + (size_t)t * C + 8 * i) = d.p[p];
+        }
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -725,7 +670,7 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
     group_body<FEW>(G, s_count, s_off, reinterpret_cast<int*>(xs));     // the token row is no longer needed
     if (A.do_sched) {
         __syncthreads();
-        schedule_body(S, s_count, E + G.ns, s_off, reinterpret_cast<int*>(xs));   // s_off and xs are free now
+        schedule_body(S, s_count, E + G.ns, s_off);   // s_off is free now
     }
     if (threadIdx.x == 0) *A.ticket = 0u;
 }
@@ -743,7 +688,7 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
     __shared__ int s_rank[kSingleCtaMaxTokens][kMaxTopK];
     __shared__ int s_count[kMaxExperts];
     __shared__ int s_off[kMaxExperts + 1];
-    __shared__ int s_tb[kMaxExperts];
+    __shared__ unsigned s_word[kMaxExperts / 32];
     __shared__ int s_slot[kMaxExperts];
     const int T = A.T, C = A.C, E = A.E, k = A.k, c8 = C / 8, ns = G.ns, Etot = E + ns, kk = k + ns;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = kSingleCtaThreads / 32;
@@ -807,6 +752,11 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
                 o4[j] = *reinterpret_cast<const unsigned*>(&h);
             }
             og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+            if (A.xq != nullptr) {
+                const Digits8 d = digits_of_x16(o4);
+#pragma unroll
+                for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A.xq + p * A.xq_plane + (size_t)t * C + 8 * i) = d.p[p];
+            }
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
@@ -905,15 +855,15 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
         const int e = threadIdx.x;
         const bool need = e < Etot && s_count[e] > 0;
         const bool res = need && s_slot[e] >= 0;
-        s_tb[e] = res ? (s_count[e] + kTokBlock - 1) / kTokBlock : 0;
         const unsigned done = __ballot_sync(0xffffffffu, res), miss = __ballot_sync(0xffffffffu, need && !res);
         if (lane == 0) {
             S.done_mask[e >> 5] = done;
+            s_word[e >> 5] = done;
             if (miss && !S.quiet) { atomicOr(S.miss_mask + (e >> 5), miss); atomicOr(S.status, 1); }
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) write_schedule(S.sched, s_tb, s_count, Etot, S.tc_min[0], S.tc_min[1]);
+    write_schedule(S, s_word);
 }
 
 // S7 pooling of per-token scores that the caller asked for: pooled[e] = mean_t score[t][e]; then the k_pred best.
@@ -1058,7 +1008,7 @@ SchedArgs sched_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map,
                      bool quiet = false) {
     SchedArgs S;
     S.quiet = quiet ? 1 : 0;
-    S.slots = slots; S.hexp = ws_ptr<int32_t>(ctx, ctx->lay.hexp);
+    S.slots = slots; S.hexp = ws_ptr<int32_t>(ctx, ctx->lay.hexp); S.wmaps = ws_ptr<unsigned char>(ctx, ctx->lay.wmaps);
     S.T = T; S.R = ctx->cfg.ffn; S.C = ctx->cfg.hidden; S.per_matrix = ctx->cfg.format == MIRA_FORMAT_PER_MATRIX; S.n_main = n_main;
     step_tc_min(ctx, T, k, S.tc_min);
     const int Etot = Et(ctx->cfg);
@@ -1090,6 +1040,8 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
         A.k = k; A.idx = rv.idx; A.wts = rv.w;
         A.ticket = ws_ptr<unsigned>(ctx, ctx->lay.status) + 8;
         A.do_sched = slot_map != nullptr;
+        A.xq = T <= kTokenOrderMax ? ws_ptr<int8_t>(ctx, ctx->lay.xq) : nullptr;
+        A.xq_plane = (size_t)Pmax(ctx->cfg) * C;
         SchedArgs S = sched_args(ctx, slots, slot_map, nullptr, T, k, single ? 1 : T, quiet_schedule);
         ProfScope ps(ctx, MIRA_K_ROUTE, st);
         if (single) MIRA_CUDA_OK(launch_pdl(k_route_small, dim3(1 + n_stat), dim3(kSingleCtaThreads), (size_t)T * C * 2, st, A, G, S));
