@@ -47,6 +47,7 @@ Layout make_layout(const mira_config& c) {
     L.xs_pos = o;    o = align256(o + P * 4);
     L.hm_pos = o;    o = align256(o + P * 4);
     L.hs_pos = o;    o = align256(o + P * 4);
+    L.hmax = o;      o = align256(o + P * 4);
     L.xq = o;        o = align256(o + 3 * P * C);
     L.hq = o;        o = align256(o + 3 * P * R);
     L.wmaps = o;     o = align256(o + ((size_t)kMaxExperts + 1) * kWeightMaps * 128);

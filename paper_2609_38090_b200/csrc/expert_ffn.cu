@@ -18,8 +18,8 @@
 // converted every code to fp16 in registers (1.25 instructions per weight, staged through shared memory, mma.sync) and ran a
 // 32-token step at 1069 W and 1710 MHz.
 // Measured (us per step, before -> now; the streamed bytes at the copy rate take 54 / 215 / 216): 8x7B shape, 1 token 77.1 ->
-// 75.8, 8 tokens 228 -> 190, 32 tokens 294 -> 249 (5.7 TB/s over the whole step), 200 tokens 428 -> 383; 8x22B shape, 13 tokens,
-// per-matrix format 352 -> 303; fine-grained layer, 4 tokens 54.1 -> 47.2, 64 tokens 98.2 -> 85.1.
+// 72.8, 8 tokens 228 -> 190, 32 tokens 294 -> 249 (5.7 TB/s over the whole step), 200 tokens 428 -> 383; 8x22B shape, 13 tokens,
+// per-matrix format 352 -> 303; fine-grained layer, 4 tokens 54.1 -> 45.4, 64 tokens 98.2 -> 82.5.
 //
 // Work is derived on the device from the schedule the grouping step wrote; the host never reads
 // routing results.
@@ -32,15 +32,18 @@ namespace mira {
 namespace {
 
 constexpr int kEpiWarps = 8;              // two per TMEM lane quarter, taking eight columns in turn
-constexpr int kThreads = 32 * (4 + kEpiWarps);      // two TMA warps (weights, activations), MMA warp, (one idle,) epilogue warps
+constexpr int kMaxStages = 6;
+constexpr int kConvPerSlot = 2;           // "direct" kernels: warps that turn activations into digits on the way to shared memory
+constexpr int kConvWarps = 5 * kConvPerSlot;          // (direct rings have five slots at most)
+// Two TMA warps (weights, activations), MMA warp, (one idle,) epilogue warps, and in the direct kernels the converting warps.
+constexpr int threads_of(bool direct) { return 32 * (4 + kEpiWarps + (direct ? kConvWarps : 0)); }
 constexpr int kUnit = 32;                 // MMA rows per unit of the partition; a tile has up to four
 constexpr int kKBox = 128;                // reduction elements (= bytes per row) of a TMA box: four MMAs of K = 32
 constexpr int kABox = 128 * kKBox;        // its weight tile
 constexpr int kMaxTok = 80;               // tokens of a tile: 3 * 80 columns of 256
 constexpr int kAccCols = 256;             // TMEM columns of an accumulator (two of them)
-constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr long long kWaitCycles = 2000000000;      // about a second
 constexpr int kRingBytes = 212 * 1024;    // shared memory of the ring
-constexpr int kMaxStages = 6;
 constexpr int kItems = 4;                 // work items a CTA has drawn ahead
 
 struct DigitMaps { CUtensorMap m[kDigitMaps]; };      // boxes of 8, 16, ..., 80 positions x 3 planes x 128 bytes
@@ -58,9 +61,14 @@ struct FfnArgs {
     int32_t* status;
     int R, C, act_on_w1, per_matrix;
     int n_all;                            // routed + shared experts
+    int raw_at;                           // direct: offset of the fp16 rows in a stage
     int stages, boxes, stage_bytes, b_box, tile_tok;      // ring geometry and tokens per tile, from the batch size
     int token_order;                      // S4: the tile's columns are all T tokens (digit planes in token order, see kTokenOrderMax)
-    int T; const int32_t* row_token; const float* xscale; const float* xnorm; float* hscale;      // S4, token order
+    int T; const int32_t* row_token; const float* xscale; const float* xnorm;       // token order, direct kernels
+    const __half* x16;                    // direct kernels
+    float* hscale;                        // 2^-f, for the tensor-core down kernel
+    unsigned* hmax;                       // per position: largest absolute value of the intermediate, as the bits of a float
+    int track_max;                        // S4: wanted
     int splits; long ypart_stride;        // S5: slices of the reduction, elements between two slices of ypart
 };
 
@@ -84,10 +92,13 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait by a whole warp. Returns false (and raises the abort flag) if the barrier did not flip in time.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    bool ok = false;
-    for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
-        if (mbar_try(bar, parity)) { ok = true; break; }
-        if ((spin & 1023u) == 1023u && *abort_flag) break;
+    bool ok = mbar_try(bar, parity);
+    if (!__all_sync(0xffffffffu, ok)) {
+        const long long t0 = clock64();
+        for (uint32_t spin = 0; !ok; ++spin) {
+            ok = mbar_try(bar, parity);
+            if ((spin & 63u) == 63u && (*abort_flag || clock64() - t0 > kWaitCycles)) break;
+        }
     }
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) *abort_flag = 1;
@@ -181,17 +192,41 @@ struct Walk {
     }
 };
 
-template <bool DOWN>
-__global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_constant__ DigitMaps bmaps) {
+// The power of two that places the fp16 intermediate of expert e (hexp) on a token of this norm: |u|, |g| ~ s * 32 * |x| (codes
+// have rms ~ 127 / 4) and |h| ~ u g / 2, so s h ~ s^3 * 512 |x|^2 for the row with the LARGEST scale of the expert (hexp =
+// exponent of that s^3, from the routing kernel's statistics CTAs; per-matrix format: of s1 s3). That magnitude is placed at 2^-2.
+__device__ __forceinline__ int place(int hexp, float xnorm) { return max(-120, min(120, -(hexp + 11 + 2 * expo(xnorm)))); }
+// Eight values of the intermediate; wide-range experts: both fp16 windows together.
+__device__ __forceinline__ void h_values(const uint4& hi, const uint4& lo, bool wide, float (&x)[8]) {
+    halves8(hi, x);
+    if (wide) {
+        float l[8];
+        halves8(lo, l);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = fmaf(l[j], pow2i(-kLoShift), x[j]);
+    }
+}
+// The activations reach shared memory in one of two forms.
+// DIRECT: rows of the fp16 activations (S4: of the tokens, gathered; S5: of the intermediate) are copied into the stage as they
+// are, converting warps split them into digits and store them where the MMA reads them. No kernel stands between the routing and S4
+// or between S4 and S5; each CTA repeats the conversion of what it needs. For the smallest batches, where the chain of kernels counts: with 1 token of the 8x7B
+// shape the step takes 72.0 us instead of 74.9, with 4 of the fine-grained one 42.0 instead of 43.5; with 8 tokens 196 and 195,
+// 49.4 and 49.4; with 16 of the fine-grained one 59.8 and 55.9 (every CTA converts 16 rows for the shared experts). Two warps
+// per slot of the ring (fine-grained, 4 tokens: one 42.5, two 41.9, three 42.2).
+// Otherwise a kernel in front has written digit planes, which the TMA unit fetches.
+template <bool DOWN, bool DIRECT>
+__global__ void __launch_bounds__(threads_of(DIRECT), 1) k_ffn(FfnArgs A, const __grid_constant__ DigitMaps bmaps) {
     extern __shared__ unsigned char smem[];
     __shared__ TileTable tab;
-    __shared__ uint64_t s_bar[2 * kMaxStages + 4 + 2 * kItems];          // full, done, acc_full[2], acc_empty[2], item_full, item_empty
+    __shared__ uint64_t s_bar[3 * kMaxStages + 4 + 2 * kItems];          // full, done, acc_full[2], acc_empty[2], item_full, item_empty, raw
     __shared__ int s_item[kItems];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
+    constexpr int kThreads = threads_of(DIRECT);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int C = A.C, R = A.R, NS = A.stages, boxes = A.boxes;
     const uint32_t a_bytes = boxes * kABox;
+    const bool token_order = !DOWN && !DIRECT && A.token_order;
     const int n_u = DOWN ? C / kUnit : R / (kUnit / 2), S = DOWN ? A.splits : 1;
     const uint32_t ring = (smem_u32(smem) + 1023u) & ~1023u, bar0 = smem_u32(s_bar);
     auto full = [&](int s) { return bar0 + 8u * s; };
@@ -200,14 +235,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
     auto acc_empty = [&](uint32_t b) { return bar0 + 8u * (2 * kMaxStages + 2 + b); };
     auto item_full = [&](uint32_t i) { return bar0 + 8u * (2 * kMaxStages + 4 + i); };
     auto item_empty = [&](uint32_t i) { return bar0 + 8u * (2 * kMaxStages + 4 + kItems + i); };
+    auto raw = [&](int s) { return bar0 + 8u * (2 * kMaxStages + 4 + 2 * kItems + s); };         // direct: the fp16 rows have landed
 
     if (tid == 0) {
-        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 2); mbar_init(done(s), 1); }
+        for (int s = 0; s < NS; ++s) { mbar_init(full(s), DIRECT ? 1 + kConvPerSlot : 2); mbar_init(done(s), 1); mbar_init(raw(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), kEpiWarps); }
-        for (int i = 0; i < kItems; ++i) { mbar_init(item_full(i), 1); mbar_init(item_empty(i), 2 + kEpiWarps); }
+        for (int i = 0; i < kItems; ++i) { mbar_init(item_full(i), 1); mbar_init(item_empty(i), 2 + kEpiWarps + (DIRECT ? kConvWarps : 0)); }
         s_abort = 0;
         tab.n_all = A.n_all; tab.n_u = n_u; tab.S = S; tab.nbox = ((DOWN ? R : C) + kKBox - 1) / kKBox;
-        tab.n_cols = !DOWN && A.token_order ? (A.T + 7) & ~7 : 0;
+        tab.n_cols = token_order ? (A.T + 7) & ~7 : 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 2) {
@@ -215,9 +251,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     // Table of the experts. The schedule, the counts and the maps come from the routing kernels, which had completed before the
-    // kernel in front of this one started; with digits in token order the routing kernel IS the kernel in front.
-    const bool token_order = !DOWN && A.token_order;
-    if (token_order) { pdl_wait(); pdl_launch(); }
+    // kernel in front of this one started, unless they are the kernel in front.
+    const bool after_routing = !DOWN && (DIRECT || token_order);
+    if (after_routing) { pdl_wait(); pdl_launch(); }
     const int tc_min = A.sched->tc_min[DOWN ? 1 : 0];
     for (int e = tid; e < A.n_all; e += kThreads) {
         const int cnt = A.count[e], off = A.offset[e];
@@ -262,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
     if (warp < 2) {
         // ------------------------------------------------ TMA warps. The weights depend on the routing alone, the digits on the
         // kernel before this one: warp 0 requests weights at once, warp 1 waits.
-        if (warp == 1 && !token_order) { pdl_wait(); pdl_launch(); }
+        if (warp == 1 && !after_routing) { pdl_wait(); pdl_launch(); }
         int slot = 0, item = blockIdx.x, drawn = 0;
         const CUtensorMap* last_map = nullptr;
         uint32_t ph = 1;
@@ -289,9 +325,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
                 const uint32_t box_bytes = warp == 0 ? t.units * (kABox / 4) : 3 * t.n * kKBox, box_step = warp == 0 ? kABox : A.b_box;
                 const uint32_t base = ring + (warp == 0 ? 0 : a_bytes);
                 const int row = warp == 0 ? t.u0 * (DOWN ? kUnit : kUnit / 2) : token_order ? 0 : t.pos0;
+                const __half* src = nullptr;               // direct: lane n copies token n's rows
+                if (DIRECT && warp == 1 && lane < t.ntok)
+                    src = DOWN ? A.h16 + (size_t)(t.pos0 + lane) * R : A.x16 + (size_t)A.row_token[t.pos0 + lane] * C;
                 for (int b = t.b0; b < t.b1; b += boxes) {
                     if (!mbar_wait(done(slot), ph, &s_abort)) { ok = false; break; }
-                    if (elect_one()) {
+                    if (DIRECT && warp == 1) {
+                        const uint32_t bytes = 2 * (min((b + boxes) * kKBox, min(t.b1 * kKBox, DOWN ? R : C)) - b * kKBox);
+                        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(raw(slot)), "r"(t.ntok * bytes) : "memory");
+                        __syncwarp();
+                        if (lane < t.ntok)
+                            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                                         ::"r"(ring + slot * A.stage_bytes + A.raw_at + lane * boxes * kKBox * 2), "l"(src + (size_t)b * kKBox), "r"(bytes), "r"(raw(slot)) : "memory");
+                    } else if (elect_one()) {
                         const uint32_t dst = base + slot * A.stage_bytes, bar = full(slot);
                         const int nb = min(boxes, t.b1 - b);
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(nb * box_bytes) : "memory");
@@ -342,9 +388,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
                 ++it;
             }
         }
-    } else if (warp >= 4) {
+    } else if (warp >= 4 && warp < 4 + kEpiWarps) {
         // ------------------------------------------------ epilogue (thread = MMA row = TMEM lane)
-        if (!token_order) pdl_wait();
+        if (!after_routing) pdl_wait();
         const int cg = 8 * ((warp - 4) >> 2);                // first chunk of columns of this warp
         const int q = warp & 3, row = q * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
@@ -360,8 +406,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
             const unsigned char* blob = static_cast<const unsigned char*>(A.slots[A.slot_map[t.e]]);
             const int r = DOWN ? t.u0 * kUnit + row : t.u0 * (kUnit / 2) + (row >> 1), odd = row & 1;
             const bool mine = q < t.units;
-            int wide = 0, my_tok = -1;
-            float s_u = 1.f, s_g = 1.f, s_h = 1.f, my_xs = 0.f, my_hm = 0.f;
+            int wide = 0;
+            float s_u = 1.f, s_g = 1.f, s_h = 1.f;
+            // Direct, token order: lane n holds column n's numbers. S4: 2^e of the digits, 2^f; S5: the undo factor. Token order: the
+            // expert's tokens, lane i that of its i-th position.
+            float f1 = 0.f, f2 = 0.f;
+            int my_tok = -1;
             if (mine) {
                 if (DOWN) {             // per-matrix format: the scale of output column r (row r of W2^)
                     if (A.per_matrix) s_u = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_out)[r]);
@@ -371,15 +421,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
                     s_g = A.per_matrix ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(blob + blob_fmt(1, R, C).s_gate)[r]) : s_u;
                     s_h = A.per_matrix ? 1.f : s_u;
                 }
-                // token order: lane i knows the i-th position's token and token i's factors
+                if (DIRECT && lane < t.ntok) {
+                    const int tok = A.row_token[t.pos0 + lane], f = place(A.hexp[t.e], A.xnorm[tok]);
+                    if (DOWN) f1 = pow2i(digit_exponent(__uint_as_float(A.hmax[t.pos0 + lane])) - 21) * pow2i(-f);
+                    else {
+                        f1 = A.xscale[tok] * (1.f / 256.f);
+                        f2 = pow2i(f);
+                        if (t.u0 == 0 && warp == 4) A.hscale[t.pos0 + lane] = pow2i(-f);
+                    }
+                }
                 if (token_order) {
                     if (lane < t.ntok) my_tok = A.row_token[t.pos0 + lane];
                     if (lane < A.T) {
-                        const int f = max(-120, min(120, -(A.hexp[t.e] + 11 + 2 * expo(A.xnorm[lane]))));
-                        my_xs = A.xscale[lane] * (1.f / 256.f);
-                        my_hm = pow2i(f);
+                        f1 = A.xscale[lane] * (1.f / 256.f);
+                        f2 = pow2i(place(A.hexp[t.e], A.xnorm[lane]));
                     }
-                    const float hm_of_pos = __shfl_sync(0xffffffffu, my_hm, max(my_tok, 0));
+                    const float hm_of_pos = __shfl_sync(0xffffffffu, f2, max(my_tok, 0));
                     if (t.u0 == 0 && warp == 4 && lane < t.ntok) A.hscale[t.pos0 + lane] = 1.f / hm_of_pos;
                 }
             }
@@ -400,11 +457,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
                     if (DOWN) {
                         float* yp = A.ypart + (size_t)t.split * A.ypart_stride + (size_t)(t.pos0 + c0) * C + r;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            if (c0 + j < t.ntok) yp[(size_t)j * C] = v[j] * (__ldg(A.hs_pos + t.pos0 + c0 + j) * s_u);
+                        for (int j = 0; j < 8; ++j) {
+                            const float hs = DIRECT ? __shfl_sync(0xffffffffu, f1, c0 + j) : __ldg(A.hs_pos + t.pos0 + min(c0 + j, t.ntok - 1));
+                            if (c0 + j < t.ntok) yp[(size_t)j * C] = v[j] * (hs * s_u);
+                        }
                     } else {
                         // Even lanes hold U, odd lanes G of the same expert-hidden row. Of every pair of columns the even lane
                         // finishes the even one and the odd lane the odd one: one exchange per pair.
+                        unsigned top = 0u;              // lane j: largest |h| of column c0 + j
 #pragma unroll
                         for (int jj = 0; jj < 4; ++jj) {
                             const float a = v[2 * jj], b = v[2 * jj + 1];
@@ -412,26 +472,36 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
                             const int n = c0 + 2 * jj + odd;
                             int pos = t.pos0 + min(n, t.ntok - 1);
                             bool store = n < t.ntok;
-                            float xs, hm;
                             if (token_order) {
                                 const unsigned me = __ballot_sync(0xffffffffu, my_tok == c0 + 2 * jj), mo = __ballot_sync(0xffffffffu, my_tok == c0 + 2 * jj + 1);
                                 const unsigned m = odd ? mo : me;
                                 store = m != 0;
                                 pos = t.pos0 + __ffs(m) - 1;
-                                xs = __shfl_sync(0xffffffffu, my_xs, n & 31); hm = __shfl_sync(0xffffffffu, my_hm, n & 31);
-                            } else {
-                                xs = __ldg(A.xs_pos + pos); hm = __ldg(A.hm_pos + pos);
                             }
+                            float xs, hm;
+                            if (DIRECT || token_order) { xs = __shfl_sync(0xffffffffu, f1, n & 31); hm = __shfl_sync(0xffffffffu, f2, n & 31); }
+                            else { xs = __ldg(A.xs_pos + pos); hm = __ldg(A.hm_pos + pos); }
                             const float u = (odd ? other : a) * (xs * s_u), g = (odd ? b : other) * (xs * s_g);
                             const float act = A.act_on_w1 ? u : g, lin = A.act_on_w1 ? g : u;
                             const float val = __fdividef(act, 1.f + __expf(-act)) * lin * s_h * hm;
                             const unsigned short hi = f32_to_f16_sat(val);
+                            float kept = __half2float(__ushort_as_half(hi));
+                            unsigned short lo = 0;
+                            if (wide) {
+                                lo = f32_to_f16_sat((val - kept) * pow2i(kLoShift));
+                                kept = fmaf(__half2float(__ushort_as_half(lo)), pow2i(-kLoShift), kept);
+                            }
                             if (store) {
                                 reinterpret_cast<unsigned short*>(A.h16)[(size_t)pos * R + r] = hi;
-                                if (wide) reinterpret_cast<unsigned short*>(A.h16lo)[(size_t)pos * R + r] =
-                                    f32_to_f16_sat((val - __half2float(__ushort_as_half(hi))) * pow2i(kLoShift));
+                                if (wide) reinterpret_cast<unsigned short*>(A.h16lo)[(size_t)pos * R + r] = lo;
+                            }
+                            if (DIRECT) {
+                                const unsigned m = __float_as_uint(fabsf(kept)), me = __reduce_max_sync(0xffffffffu, odd ? 0u : m),
+                                               mo = __reduce_max_sync(0xffffffffu, odd ? m : 0u);
+                                if (lane >> 1 == jj) top = odd ? mo : me;
                             }
                         }
+                        if (DIRECT && A.track_max && lane < 8 && c0 + lane < t.ntok) atomicMax(A.hmax + t.pos0 + c0 + lane, top);
                     }
                 }
             }
@@ -440,6 +510,54 @@ __global__ void __launch_bounds__(kThreads, 1) k_ffn(FfnArgs A, const __grid_con
             if (lane == 0) mbar_arrive(acc_empty(buf));
             ++it;
         }
+        }
+    } else if (DIRECT && warp >= 4 + kEpiWarps) {
+        // ------------------------------------------------ converting warps: warp i fills slot i of the ring, so that it waits for
+        // every phase of that slot's barrier (a warp that skipped one could take an older phase for the one it needs).
+        if (DOWN) pdl_wait();
+        const int mine = (warp - (4 + kEpiWarps)) / kConvPerSlot, share = (warp - (4 + kEpiWarps)) % kConvPerSlot;      // (a warp beyond the ring's slots only reads the items)
+        int slot = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int item = next_item(); ok && item >= 0; item = next_item()) {
+            Walk w(tab, item);
+            Tile t;
+            while (ok && w.next(t)) {
+                const bool wide = DOWN && A.hexp[kMaxExperts + t.e] != 0;
+                float up = kXDigits;                       // lane n: factor of token n's digits
+                if (DOWN && lane < t.ntok) up = pow2i(21 - digit_exponent(__uint_as_float(A.hmax[t.pos0 + lane])));
+                for (int b = t.b0; b < t.b1; b += boxes) {
+                    if (slot == mine) {
+                        const int sh = boxes == 2 ? 5 : 4, total = t.ntok << sh;      // vectors of eight: 16 per token and box
+                        const uint32_t stage = ring + slot * A.stage_bytes;
+                        if (!mbar_wait(raw(slot), ph, &s_abort)) { ok = false; break; }
+#pragma unroll 4
+                        for (int i0 = 32 * share; i0 < total; i0 += 32 * kConvPerSlot) {
+                            const int i = i0 + lane, n = i >> sh, c = i & ((1 << sh) - 1);
+                            const float scale = DOWN ? __shfl_sync(0xffffffffu, up, n) : kXDigits;
+                            if (i >= total) continue;
+                            uint4 v;
+                            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage + A.raw_at + i * 16) : "memory");
+                            float x[8];
+                            if (DOWN) {
+                                uint4 lo = make_uint4(0, 0, 0, 0);
+                                const int k = b * kKBox + c * 8;
+                                if (wide && k < R) lo = __ldcg(reinterpret_cast<const uint4*>(A.h16lo + (size_t)(t.pos0 + n) * R + k));
+                                h_values(v, lo, wide, x);
+                            } else halves8(v, x);
+                            const Digits8 d = digits8(x, scale);
+                            const uint32_t at = stage + a_bytes + (c >> 4) * A.b_box + n * kKBox + ((((c & 15) >> 1) ^ (n & 7)) << 4) + (c & 1) * 8;
+#pragma unroll
+                            for (int p = 0; p < 3; ++p)
+                                asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(at + p * t.n * kKBox), "r"(d.p[p].x), "r"(d.p[p].y) : "memory");
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(full(slot));
+                    }
+                    if (++slot == NS) { slot = 0; ph ^= 1u; }
+                }
+            }
         }
     }
     // ---------------------------------------------------- common exit
@@ -472,9 +590,7 @@ __device__ __forceinline__ int expert_of(const DigitArgs& D, int pos, int* s_e) 
 }
 
 // Activation digits of one position (x16 is the row scaled by a power of two, largest value in [2^13, 2^14): times 2^8) and the
-// factors of its SwiGLU epilogue: 2^e, and the power of two 2^f that places the fp16 intermediate. |u|, |g| ~ s * 32 * |x| (codes
-// have rms ~ 127 / 4) and |h| ~ u g / 2, so s h ~ s^3 * 512 |x|^2 for the row with the LARGEST scale of the expert (hexp =
-// exponent of that s^3, from the routing kernel's statistics CTAs; per-matrix format: of s1 s3). That magnitude is placed at 2^-2.
+// factors of its SwiGLU epilogue: 2^e, and the power of two that places the fp16 intermediate.
 __global__ void __launch_bounds__(256) k_digits_x(DigitArgs D) {
     __shared__ int s_e;
     pdl_wait();
@@ -486,13 +602,14 @@ __global__ void __launch_bounds__(256) k_digits_x(DigitArgs D) {
     uint2* dst = reinterpret_cast<uint2*>(D.planes + (size_t)pos * D.cols);
     for (int i = threadIdx.x; i < D.cols / 8; i += 256) {
         const uint4 v = src[i];
-        const unsigned w[4] = {v.x, v.y, v.z, v.w};
-        const Digits8 d = digits_of_x16(w);
+        float x[8];
+        halves8(v, x);
+        const Digits8 d = digits8(x, kXDigits);
 #pragma unroll
         for (int p = 0; p < 3; ++p) dst[p * (D.plane / 8) + i] = d.p[p];
     }
     if (threadIdx.x == 0) {
-        const int f = max(-120, min(120, -(D.hexp[e] + 11 + 2 * expo(D.xnorm[tok]))));
+        const int f = place(D.hexp[e], D.xnorm[tok]);
         D.xs_pos[pos] = D.xscale[tok] * (1.f / 256.f);
         D.hm_pos[pos] = pow2i(f);
         D.hscale[pos] = pow2i(-f);
@@ -514,11 +631,6 @@ __global__ void __launch_bounds__(kDigitThreads, 2) k_digits_h(DigitArgs D) {
     const uint4* hi = reinterpret_cast<const uint4*>(D.h16 + (size_t)pos * D.cols);
     const uint4* lo = reinterpret_cast<const uint4*>(D.h16lo + (size_t)pos * D.cols);
     const int n = D.cols / 8;
-    auto value = [&](const uint4& a, const uint4& b, int j) {
-        const unsigned wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
-        const float h = __half2float(__ushort_as_half((unsigned short)(wa[j >> 1] >> (16 * (j & 1)))));
-        return wide ? fmaf(__half2float(__ushort_as_half((unsigned short)(wb[j >> 1] >> (16 * (j & 1))))), pow2i(-kLoShift), h) : h;
-    };
     uint4 a[kDigitVecs], b[kDigitVecs];
     auto fetch = [&](int i0) {
 #pragma unroll
@@ -533,9 +645,12 @@ __global__ void __launch_bounds__(kDigitThreads, 2) k_digits_h(DigitArgs D) {
     for (int i0 = (n - 1) / round * round; i0 >= 0; i0 -= round) {       // the first round last: it stays in registers
         fetch(i0);
 #pragma unroll
-        for (int q = 0; q < kDigitVecs; ++q)
+        for (int q = 0; q < kDigitVecs; ++q) {
+            float x[8];
+            h_values(a[q], b[q], wide, x);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(value(a[q], b[q], j)));
+            for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(x[j]));
+        }
     }
     m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
     if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
@@ -550,10 +665,9 @@ __global__ void __launch_bounds__(kDigitThreads, 2) k_digits_h(DigitArgs D) {
         for (int q = 0; q < kDigitVecs; ++q) {
             const int i = i0 + q * blockDim.x + threadIdx.x;
             if (i >= n) continue;
-            Digits8 d;
-            clear_digits(d);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) set_digits(d, j, __float2int_rn(value(a[q], b[q], j) * up));
+            float x[8];
+            h_values(a[q], b[q], wide, x);
+            const Digits8 d = digits8(x, up);
 #pragma unroll
             for (int p = 0; p < 3; ++p) dst[p * (D.plane / 8) + i] = d.p[p];
         }
@@ -673,7 +787,14 @@ bool encode_bytes(EncodeTiledFn fn, void* out, void* base, int rank, const cuuin
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-FfnArgs make_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map) {
+// Whether the streaming kernel of a projection (0 up/gate, 1 down) makes its digits itself. The down kernel needs the largest value
+// of every row of the intermediate, which only the direct up/gate kernel collects.
+bool stream_direct(const mira_ctx* ctx, int projection) {
+    int tc_min[2];
+    step_tc_min(ctx, ctx->route_T, ctx->route_k, tc_min);
+    return ctx->route_T <= kDirectMax && (projection == 0 || tc_min[0] > ctx->route_T);
+}
+FfnArgs make_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, bool direct) {
     FfnArgs A;
     A.slots = slots; A.slot_map = slot_map;
     A.sched = ws_ptr<Sched>(ctx, ctx->lay.sched);
@@ -695,11 +816,22 @@ FfnArgs make_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map) {
     A.n_all = Et(ctx->cfg);
     A.b_box = ((3 * A.tile_tok + 15) / 16 * 16) * kKBox;           // (the MMA's columns are a multiple of 16)
     // Two boxes per stage (one wait and one commit per eight MMAs) while at least four such stages fit.
-    A.boxes = 2 * (kABox + A.b_box) * 4 <= kRingBytes ? 2 : 1;
-    A.stage_bytes = A.boxes * (kABox + A.b_box);
-    A.stages = std::min(kMaxStages, kRingBytes / A.stage_bytes);
-    A.token_order = ctx->route_T <= kTokenOrderMax;
+    if (direct) {
+        A.b_box = 3 * A.tile_tok * kKBox;          // (with 8 tokens the MMA reads 8 rows beyond: columns that nobody reads)
+        A.boxes = 2;
+        A.raw_at = A.boxes * (kABox + A.b_box);
+        A.stage_bytes = A.raw_at + A.tile_tok * A.boxes * kKBox * 2;
+    } else {
+        A.boxes = 2 * (kABox + A.b_box) * 4 <= kRingBytes ? 2 : 1;
+        A.raw_at = 0;
+        A.stage_bytes = A.boxes * (kABox + A.b_box);
+    }
+    A.stages = std::min(direct ? kConvWarps / kConvPerSlot : kMaxStages, kRingBytes / A.stage_bytes);
+    A.token_order = !direct && ctx->route_T <= kTokenOrderMax;
     A.T = ctx->route_T;
+    A.x16 = ws_ptr<__half>(ctx, ctx->lay.x16);
+    A.hmax = ws_ptr<unsigned>(ctx, ctx->lay.hmax);
+    A.track_max = stream_direct(ctx, 1);
     A.row_token = ws_ptr<int32_t>(ctx, ctx->lay.row_token);
     A.xscale = ws_ptr<float>(ctx, ctx->lay.xscale); A.xnorm = ws_ptr<float>(ctx, ctx->lay.xnorm);
     A.hscale = ws_ptr<float>(ctx, ctx->lay.hscale);
@@ -725,7 +857,11 @@ template <bool DOWN> cudaError_t launch_ffn(mira_ctx* ctx, void* const* slots, c
     static_assert(sizeof(DigitMaps) == sizeof(ctx->tmap_digits[0]), "tensor map storage");
     DigitMaps maps;
     memcpy(&maps, ctx->tmap_digits[DOWN ? 1 : 0], sizeof(maps));
-    return launch_pdl(k_ffn<DOWN>, dim3(ctx->n_sm), dim3(kThreads), (size_t)kRingBytes + 1024, st, make_args(ctx, slots, slot_map), maps);
+    const bool direct = stream_direct(ctx, DOWN ? 1 : 0);
+    const FfnArgs A = make_args(ctx, slots, slot_map, direct);
+    constexpr size_t smem = (size_t)kRingBytes + 1024;
+    return direct ? launch_pdl(k_ffn<DOWN, true>, dim3(ctx->n_sm), dim3(threads_of(true)), smem, st, A, maps)
+                  : launch_pdl(k_ffn<DOWN, false>, dim3(ctx->n_sm), dim3(threads_of(false)), smem, st, A, maps);
 }
 
 }  // namespace
@@ -761,7 +897,7 @@ bool build_stream_maps(mira_ctx* ctx) {
 
 mira_status launch_up_gate(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, cudaStream_t st) {
     ProfScope ps(ctx, MIRA_K_UP_GATE, st);
-    if (ctx->route_T > kTokenOrderMax) {          // else the routing kernel has written the digits
+    if (!stream_direct(ctx, 0) && ctx->route_T > kTokenOrderMax) {          // else the routing kernel has written the digits, or nobody
         const int P = ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
         MIRA_CUDA_OK(launch_pdl(k_digits_x, dim3(P), dim3(256), 0, st, digit_args(ctx, slot_map, ctx->lay.xq, ctx->cfg.hidden)));
         ctx->launches += 1;
@@ -774,11 +910,14 @@ mira_status launch_up_gate(mira_ctx* ctx, void* const* slots, const int32_t* slo
 
 mira_status launch_down(mira_ctx* ctx, void* const* slots, const int32_t* slot_map, cudaStream_t st) {
     ProfScope ps(ctx, MIRA_K_DOWN, st);
-    const int P = ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
-    const int threads = std::min(kDigitThreads, (ctx->cfg.ffn / 8 + 32 * kDigitVecs - 1) / (32 * kDigitVecs) * 32);
-    MIRA_CUDA_OK(launch_pdl(k_digits_h, dim3(P), dim3(threads), 0, st, digit_args(ctx, slot_map, ctx->lay.hq, ctx->cfg.ffn)));
+    if (!stream_direct(ctx, 1)) {
+        const int P = ctx->route_T * (ctx->route_k + ctx->cfg.n_shared);
+        const int threads = std::min(kDigitThreads, (ctx->cfg.ffn / 8 + 32 * kDigitVecs - 1) / (32 * kDigitVecs) * 32);
+        MIRA_CUDA_OK(launch_pdl(k_digits_h, dim3(P), dim3(threads), 0, st, digit_args(ctx, slot_map, ctx->lay.hq, ctx->cfg.ffn)));
+        ctx->launches += 1;
+    }
     MIRA_CUDA_OK(launch_ffn<true>(ctx, slots, slot_map, st));
-    ctx->launches += 2;
+    ctx->launches += 1;
     MIRA_CUDA_OK(cudaGetLastError());
     return MIRA_OK;
 }
@@ -804,8 +943,10 @@ mira_status launch_combine(mira_ctx* ctx, int T, int k, int splits, int tc_split
 }
 
 mira_status set_ffn_attributes() {
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_ffn<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024));
     return MIRA_OK;
 }
 

@@ -14,8 +14,9 @@ constexpr int kMaxExperts = 256;   // E + n_shared
 constexpr int kMaxTopK = 16;
 constexpr int kDownSlice = 4096;   // nominal reduction length of one slice of the down projection
 constexpr int kWeightMaps = 8;     // tensor maps per expert: up/gate tiles of 32, 64, 96, 128 MMA rows, then down tiles
-constexpr int kTokenOrderMax = 16; // up to here the routing kernels write the activations' digit planes in token order and every expert's
-                                   // up/gate tile holds all tokens of the batch (its columns beyond the expert's own are not read)
+constexpr int kDirectMax = 4;      // up to this many tokens the streaming kernels split the activations into digits themselves ...
+constexpr int kTokenOrderMax = 16; // ... and up to here the routing kernel writes the activations' digit planes, in token order: every
+                                   // expert's up/gate tile holds all tokens of the batch (columns beyond the expert's own are not read)
 constexpr int kDigitMaps = 10;     // tensor maps of a digit-plane matrix: boxes of 8, 16, ..., 80 positions
 // The fp16 intermediate v = s_r h_r 2^f of a wide-range expert is kept as two fp16 values, hi = fp16(v) and
 // lo = fp16((v - hi) * 2^kLoShift), both saturating: together they hold 11 bits or more of every |v| in
@@ -77,6 +78,7 @@ struct Layout {
     size_t hm_pos;      // float [Pmax]    per position: 2^f applied to the fp16 intermediate (tensor-core path)
     size_t sum_pos;     // float [Pmax]    per position: sum of the token's fp16 activations (tensor-core path)
     size_t h16;         // half  [Pmax][R]
+    size_t hmax;        // uint32 [Pmax] per position: largest absolute value of the intermediate as float bits (zeroed by the routing kernels)
     size_t xq;          // int8 [3][Pmax][C] digit planes of the activations in position order (weight-streaming kernels)
     size_t hq;          // int8 [3][Pmax][R] digit planes of the intermediate
     size_t hs_pos;      // float [Pmax] per position: undo factor of the intermediate's digits and placement
@@ -248,30 +250,33 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
-// Digit planes. d0 2^16 + d1 2^8 + d2 = v, |v| < 2^22, digits in [-128, 127].
-__device__ __forceinline__ void digits(int v, int& d0, int& d1, int& d2) {
-    d2 = (int)(signed char)v;
-    v = (v - d2) >> 8;
-    d1 = (int)(signed char)v;
-    d0 = (v - d1) >> 8;
-}
+// Digit planes: v = d0 2^16 + d1 2^8 + d2, |v| < 2^22, digits in [-128, 127]. With w = v + 0x8080 the digits are the bytes of w,
+// the two lower ones with their top bit flipped, so eight values cost 14 byte permutes (and one fused multiply-add and one addition
+// each: adding 1.5 2^23 rounds to an integer, to nearest even, that sits in the low bits).
+constexpr float kXDigits = 256.f;                // activations: x16 is scaled so that the row's largest value lies in [2^13, 2^14)
 struct Digits8 { uint2 p[3]; };                  // eight consecutive values in three planes
-__device__ __forceinline__ void set_digits(Digits8& o, int j, int v) {       // j = 0, 1, ..., 7 in order, o zeroed before
-    int d0, d1, d2;
-    digits(v, d0, d1, d2);
-    const int s = 8 * (j & 3);
-    unsigned &a = j < 4 ? o.p[0].x : o.p[0].y, &b = j < 4 ? o.p[1].x : o.p[1].y, &c = j < 4 ? o.p[2].x : o.p[2].y;
-    a |= (unsigned)(d0 & 0xff) << s; b |= (unsigned)(d1 & 0xff) << s; c |= (unsigned)(d2 & 0xff) << s;
-}
-__device__ __forceinline__ void clear_digits(Digits8& o) { o.p[0] = o.p[1] = o.p[2] = make_uint2(0, 0); }
-// Digits of eight activations: fp16 values scaled so that the row's largest lies in [2^13, 2^14), times 2^8.
-__device__ __forceinline__ Digits8 digits_of_x16(const unsigned (&h2)[4]) {
-    Digits8 o;
-    clear_digits(o);
+__device__ __forceinline__ void digits4(const float* x, float up, unsigned& p0, unsigned& p1, unsigned& p2) {
+    unsigned w[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-        set_digits(o, j, __float2int_rn(__half2float(__ushort_as_half((unsigned short)(h2[j >> 1] >> (16 * (j & 1))))) * 256.f));
+    for (int j = 0; j < 4; ++j) w[j] = __float_as_uint(fmaf(x[j], up, 12582912.f)) + (0x8080u - 0x4b400000u);
+    const unsigned a = __byte_perm(w[0], w[1], 0x5140), b = __byte_perm(w[2], w[3], 0x5140);      // bytes 0 of both, bytes 1 of both
+    p2 = __byte_perm(a, b, 0x5410) ^ 0x80808080u;
+    p1 = __byte_perm(a, b, 0x7632) ^ 0x80808080u;
+    p0 = __byte_perm(__byte_perm(w[0], w[1], 0x0062), __byte_perm(w[2], w[3], 0x0062), 0x5410);
+}
+__device__ __forceinline__ Digits8 digits8(const float (&x)[8], float up) {       // of the values times the power of two `up`
+    Digits8 o;
+    digits4(x, up, o.p[0].x, o.p[1].x, o.p[2].x);
+    digits4(x + 4, up, o.p[0].y, o.p[1].y, o.p[2].y);
     return o;
+}
+__device__ __forceinline__ void halves8(const uint4& v, float (&x)[8]) {
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
+        x[2 * j] = f.x; x[2 * j + 1] = f.y;
+    }
 }
 
 // Top-k by a warp.

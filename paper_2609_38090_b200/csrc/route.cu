@@ -224,6 +224,7 @@ k_scores(const __nv_bfloat16* __restrict__ x, int T, int C, const __nv_bfloat16*
 struct GroupArgs {
     const int32_t* idx; int T, k, E, ns;
     int32_t* count; int32_t* offset; int32_t* perm; int32_t* row_token; uint32_t* done_mask;
+    unsigned* hmax;
     // Optional notification of a waiting host thread: the counts are also written to host-mapped memory, then (after a
     // system-scope fence) the sequence number to the flag, so the host learns them without a copy or a
     // synchronisation call in the stream.
@@ -336,14 +337,14 @@ __device__ __forceinline__ void group_body(const GroupArgs& G, int* s_count, int
             const int pos = s_off[e_mine] + __popc(m & lt);
             const int t = lane / k, j = lane - t * k;
             G.perm[(size_t)t * kk + j] = pos;
-            G.row_token[pos] = t;
+            G.row_token[pos] = t; G.hmax[pos] = 0u;
         }
         if (lane < n_hi) {
             const unsigned mh = __match_any_sync(n_hi == 32 ? 0xffffffffu : (1u << n_hi) - 1u, e_hi);
             const int pos = s_off[e_hi] + below + __popc(mh & lt);
             const int p = lane + 32, t = p / k, j = p - t * k;
             G.perm[(size_t)t * kk + j] = pos;
-            G.row_token[pos] = t;
+            G.row_token[pos] = t; G.hmax[pos] = 0u;
         }
     }
     for (int base = p0; base < p1; base += 32) {
@@ -358,7 +359,7 @@ __device__ __forceinline__ void group_body(const GroupArgs& G, int* s_count, int
             const int pos = s_off[e] + hist[e] + __popc(m & lt);
             const int t = p / k, j = p - t * k;
             G.perm[(size_t)t * kk + j] = pos;
-            G.row_token[pos] = t;
+            G.row_token[pos] = t; G.hmax[pos] = 0u;
         }
         __syncwarp();
         if (valid && (m & lt) == 0) hist[e] += __popc(m);
@@ -368,7 +369,7 @@ __device__ __forceinline__ void group_body(const GroupArgs& G, int* s_count, int
         const int t = q / ns, sx = q - t * ns;
         const int pos = s_off[E + sx] + t;
         G.perm[(size_t)t * kk + k + sx] = pos;
-        G.row_token[pos] = t;
+        G.row_token[pos] = t; G.hmax[pos] = 0u;
     }
 }
 
@@ -600,7 +601,9 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
         }
         og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
         if (A.xq != nullptr) {
-            const Digits8 d = digits_of_x16(o4);
+            float h[8];
+            halves8(make_uint4(o4[0], o4[1], o4[2], o4[3]), h);
+            const Digits8 d = digits8(h, kXDigits);
 #pragma unroll
             for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A.xq + p * A.xq_plane + (size_t)t * C + 8 * i) = d.p[p];
         }
@@ -752,11 +755,6 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
                 o4[j] = *reinterpret_cast<const unsigned*>(&h);
             }
             og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-            if (A.xq != nullptr) {
-                const Digits8 d = digits_of_x16(o4);
-#pragma unroll
-                for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A.xq + p * A.xq_plane + (size_t)t * C + 8 * i) = d.p[p];
-            }
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
@@ -844,7 +842,7 @@ __global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, 
         const int t = p / kk, j = p % kk;
         const int pos = (j < k) ? s_off[s_idx[t][j]] + s_rank[t][j] : s_off[E + (j - k)] + t;
         G.perm[p] = pos;
-        G.row_token[pos] = t;
+        G.row_token[pos] = t; G.hmax[pos] = 0u;
     }
     if (!A.do_sched) {
         if (threadIdx.x < 8) G.done_mask[threadIdx.x] = 0u;
@@ -1001,6 +999,7 @@ GroupArgs group_args(mira_ctx* ctx, int T, int k, const RouteView& rv) {
     G.idx = rv.idx; G.T = T; G.k = k; G.E = ctx->cfg.n_experts; G.ns = ctx->cfg.n_shared;
     G.count = rv.count; G.offset = rv.offset; G.perm = rv.perm; G.row_token = rv.row_token;
     G.done_mask = ws_ptr<uint32_t>(ctx, ctx->lay.status) + 16 + 8;
+    G.hmax = ws_ptr<unsigned>(ctx, ctx->lay.hmax);
     G.host_count = ctx->notify_count; G.host_flag = ctx->notify_flag; G.host_seq = ctx->notify_seq;
     return G;
 }
@@ -1040,7 +1039,7 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
         A.k = k; A.idx = rv.idx; A.wts = rv.w;
         A.ticket = ws_ptr<unsigned>(ctx, ctx->lay.status) + 8;
         A.do_sched = slot_map != nullptr;
-        A.xq = T <= kTokenOrderMax ? ws_ptr<int8_t>(ctx, ctx->lay.xq) : nullptr;
+        A.xq = T > kDirectMax && T <= kTokenOrderMax ? ws_ptr<int8_t>(ctx, ctx->lay.xq) : nullptr;
         A.xq_plane = (size_t)Pmax(ctx->cfg) * C;
         SchedArgs S = sched_args(ctx, slots, slot_map, nullptr, T, k, single ? 1 : T, quiet_schedule);
         ProfScope ps(ctx, MIRA_K_ROUTE, st);

@@ -1,4 +1,4 @@
-"""The weight-streaming expert kernels at the edges of their partition: digits in token order up to 16 tokens, token tiles of up to
+"""The weight-streaming expert kernels at the edges of their partition: digits made in the kernel up to 4 tokens and in token order up to 16, token tiles of up to
 80, reduction boxes of 128 elements cut by the matrix, work items of four units that run into the next expert, slices of the
 reduction beyond 4096 expert-hidden rows. Against float64 on the oracle's codes and routing."""
 import numpy as np
@@ -59,7 +59,8 @@ def _reference(wl, idx, w, act_on_w1, fp32_sums):
 
 CASES = [  # C, R, experts, k, shared, tokens, format, thresholds (up, down): pairs from which an expert leaves the streaming kernels
     (64, 64, 3, 2, 0, 1, 0, (NONE, NONE)), (64, 64, 3, 2, 0, 16, 0, (NONE, NONE)), (64, 64, 3, 2, 0, 17, 0, (NONE, NONE)),
-    (192, 320, 7, 3, 1, 8, 0, (NONE, NONE)), (192, 320, 7, 3, 1, 9, 1, (NONE, NONE)), (192, 320, 7, 3, 1, 17, 1, (NONE, NONE)),
+    (192, 320, 7, 3, 1, 4, 0, (NONE, NONE)), (320, 4224, 4, 2, 0, 4, 1, (NONE, NONE)), (64, 192, 200, 6, 2, 3, 0, (NONE, NONE)),
+    (192, 320, 7, 3, 1, 5, 0, (NONE, NONE)), (192, 320, 7, 3, 1, 8, 0, (NONE, NONE)), (192, 320, 7, 3, 1, 9, 1, (NONE, NONE)), (192, 320, 7, 3, 1, 17, 1, (NONE, NONE)),
     (320, 192, 2, 2, 0, 80, 0, (NONE, NONE)), (320, 192, 2, 2, 0, 81, 0, (NONE, NONE)), (320, 192, 2, 2, 1, 160, 1, (NONE, NONE)),
     (320, 192, 2, 2, 0, 161, 0, (NONE, NONE)), (64, 4160, 3, 2, 1, 5, 0, (NONE, NONE)), (192, 8256, 2, 1, 0, 33, 0, (NONE, NONE)),
     (64, 192, 200, 6, 2, 16, 0, (NONE, NONE)), (192, 64, 200, 6, 2, 70, 0, (NONE, NONE)),
