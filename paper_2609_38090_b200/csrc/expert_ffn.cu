@@ -155,7 +155,8 @@ struct TileTable {                // indexed by expert
     int pre[kMaxExperts + 1];     // exclusive prefix of the units (S * n_u of an expert that this kernel takes, else none)
     int n_all, n_u, S, nbox;      // experts; units per slice of the reduction, slices (S4: one), boxes of the whole reduction
     int n_cols;                   // columns per plane if every tile holds all tokens, else 0
-    int items;                    // work items: four units each
+    int items;                    // work items: four units each ...
+    int last_first;               // ... drawn from the last one on (S4: the routing kernel has asked for the shared experts' weights)
 };
 // Work is drawn item by item from a counter: bandwidth is not the same for every SM (equal shares ended 12 us apart in a 45 us
 // kernel; single-token step 84 -> 75 us). An item is four units, at 4096 reduction elements 12 us of one SM's share of HBM;
@@ -168,7 +169,7 @@ struct Walk {
     int e, u, left, nb, units;
     __device__ __forceinline__ Walk(const TileTable& table, int item) : tab(table), nb(0), units(0) {
         const int total = tab.pre[tab.n_all];
-        const int g = 4 * item;
+        const int g = 4 * (tab.last_first ? tab.items - 1 - item : item);
         left = min(4, total - g);
         int lo = 0, hi = tab.n_all - 1;                      // largest e with pre[e] <= g
         while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (tab.pre[mid] <= g) lo = mid; else hi = mid - 1; }
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(threads_of(DIRECT), 1) k_ffn(FfnArgs A, const 
         for (int i = 0; i < kItems; ++i) { mbar_init(item_full(i), 1); mbar_init(item_empty(i), 2 + kEpiWarps + (DIRECT ? kConvWarps : 0)); }
         s_abort = 0;
         tab.n_all = A.n_all; tab.n_u = n_u; tab.S = S; tab.nbox = ((DOWN ? R : C) + kKBox - 1) / kKBox;
+        tab.last_first = !DOWN;
         tab.n_cols = token_order ? (A.T + 7) & ~7 : 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
