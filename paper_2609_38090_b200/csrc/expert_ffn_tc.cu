@@ -10,10 +10,11 @@
 //             S5: 128 model-hidden rows of W2^ over the whole reduction.
 //   columns : consecutive positions of the grouping step (the tokens of one expert).
 // Warp roles, in this order:
+//   weight warp one lane loads the int8 codes by TMA, boxes of 128 rows x 128 codes (two K-blocks), through the tensor maps
+//               that the routing kernels make for every resident expert.
 //   converters  one or two groups of four warps taking K-blocks of 64 in turn. Thread t of a group owns MMA row
-//               t: the group streams its rows' int8 codes with cp.async (8 rows x 64 B per request), each thread
-//               converts its 64 codes (XOR 0x80, byte permute into the mantissa of 1024.0, subtract 1152:
-//               exact) and writes them with one tcgen05.st into the A operand ring in tensor memory (TMEM
+//               t: it reads its 64 codes from the box, converts them (XOR 0x80, byte permute into the mantissa of 1024.0,
+//               subtract 1152: exact) and writes them with one tcgen05.st into the A operand ring in tensor memory (TMEM
 //               lane = MMA row), so converted weights never touch shared memory.
 //   epilogue    four warps read the finished accumulator from TMEM, apply scales / SwiGLU, store. With two
 //               accumulators the next tile's MMAs overlap; with one, the SM's other CTA fills the gap.
@@ -28,6 +29,16 @@
 // thread pays one wait and one commit per K-block. Every wait is bounded: a wait that runs out
 // sets an error bit in the device status word and every role leaves through the common exit, where TMEM
 // is always freed.
+//
+// What bounds it: the GPU's 1000 W. A 2048-token step of the 8x7B shape ran at 1.4 GHz; with the weights copied by the converters
+// themselves (cp.async, 16 bytes a request) leaving out their copies and conversion took a quarter of its time away, the
+// conversion alone 2 to 4 %. TMA boxes move the same bytes for less energy and off the converters' chain. us per step, before
+// -> now: 8x7B 1200 tokens 1095 -> 1030, 2048: 1701 -> 1570, 3072: 2530 -> 2330; fine-grained layer 1000 tokens 328 -> 306, 256
+// tokens 144 -> 146. Left out on trial (2048 / 1000 tokens, 1625 / 318 us in that run): conversion 1556 / 307, the weights'
+// boxes too 1373 / 281, the activations' boxes 1436 / 295, tcgen05.st nothing: what moves from L2 counts most.
+// Tried and dropped: one lane that serves both rings, blocking on each in turn (3 to 10 % slower) or polling them (4 %); two
+// pairs of SMs' clusters per SM pair, so that each SM loads half of the activations (no gain: the higher clock pays for the
+// hand-overs between the SMs).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -40,11 +51,8 @@ namespace {
 
 constexpr int kTileM = 128;          // MMA rows per tile
 constexpr int kKB = 64;              // reduction elements per pipeline stage (4 MMAs of K = 16)
-constexpr int kWStages = 4;          // int8 weight ring of each converter group
 constexpr uint32_t kSpinLimit = 1u << 24;
-constexpr int kWRow = 80;            // bytes per int8 row in the weight ring: 64 + 16 pad (conflict-free row reads)
-constexpr int kWWarp = 32 * kWRow;   // one warp's 32 rows
-constexpr int kWStage = 4 * kWWarp;  // the four warps of a converter group
+constexpr int kWBox = kTileM * 128;  // weight ring: TMA boxes of 128 rows x 128 codes, two K-blocks
 
 // Kernel layout.
 //   TN      tokens per tile (at most); NS = depth of the A ring (TMEM) and of the B ring (shared memory), which share
@@ -55,27 +63,26 @@ constexpr int kWStage = 4 * kWWarp;  // the four warps of a converter group
 //   ISSUERS MMA-issuing warps (2: they take the K-blocks in turn, so one thread's barrier waits and commit overlap
 //           the other's MMAs; a turn barrier keeps the MMAs of a tile in K order)
 // TMEM columns of one CTA: ACC * TN + 32 NS, a power of two, CTAS of them in the SM's 512.
-template <int TN, int NS, int GROUPS, int ACC, int CTAS, int ISSUERS = 1, int WST = kWStages> struct TileCfg {
+template <int TN, int NS, int GROUPS, int ACC, int CTAS, int ISSUERS, int WBOXES> struct TileCfg {
     static constexpr int kTileN = TN, kStages = NS, kGroups = GROUPS, kAccBufs = ACC, kCtasPerSm = CTAS, kIssuers = ISSUERS;
-    static constexpr int kWRing = WST;           // depth of each converter group's int8 weight ring (cp.async stages)
-    static constexpr int kEpiWarp0 = 4 * GROUPS, kTmaWarp = kEpiWarp0 + 4, kMmaWarp = kEpiWarp0 + 5;
-    static constexpr int kThreads = (kMmaWarp + ISSUERS) * 32;
-    static constexpr uint32_t kTmemCols = ACC * TN + NS * 32;
+    static constexpr int kWBoxes = WBOXES;       // depth of the int8 weight ring, in boxes of two K-blocks
+    static constexpr int kEpiWarp0 = 4 * GROUPS, kTmaWarp = kEpiWarp0 + 4, kMmaWarp = kEpiWarp0 + 5, kWeightWarp = kMmaWarp + ISSUERS;
+    static constexpr int kThreads = (kWeightWarp + 1) * 32;
+    static constexpr uint32_t kTmemCols = ACC * TN + NS * 32 <= 256 ? 256 : 512;
+    static_assert(ACC * TN + NS * 32 <= 512, "TMEM columns");
     static constexpr int kBTileBytes = TN * kKB * 2;
-    static constexpr size_t kSmem = (size_t)NS * kBTileBytes + (size_t)GROUPS * WST * kWStage + 1024;
+    static constexpr size_t kSmem = (size_t)NS * kBTileBytes + (size_t)WBOXES * kWBox + 1024;
     static_assert(kTmemCols == 256 || kTmemCols == 512, "TMEM allocations are powers of two");
     static_assert(kTmemCols * CTAS <= 512, "TMEM has 512 columns per SM");
     static_assert((kSmem + 8 * 1024) * CTAS <= 227 * 1024, "shared memory per SM");
     static_assert(TN % 32 == 0, "the epilogue reads 32 columns at a time");
 };
-// Measured on the Mixtral shape (same run, us up/gate + down): 256 tokens 318 + 170 (Big) vs 261 + 118 (Narrow);
-// 1024: 580 + 342 (Big) vs 602 + 292 (Wide); 2048: 1000 + 539 (Big) vs 1035 + 469 (Wide); fine-grained shape,
-// 1024 tokens over 60 experts: 239 + 110 (Big), 228 + 104 (Wide), 211 + 97 (Narrow). The up/gate kernel has
-// short tiles with a heavy epilogue and gains from the second accumulator; the down kernel has long tiles and
-// gains from the second CTA.
-using BigTile = TileCfg<192, 4, 2, 2, 1, 2>;    // one CTA per SM, two converter groups, two accumulators, two issuers
-using WideTile = TileCfg<192, 2, 1, 1, 2>;      // two CTAs per SM
-using NarrowTile = TileCfg<128, 4, 1, 1, 2>;    // two CTAs per SM, deeper ring
+// (The big layout was the better one for many tokens per expert while the converters copied the weights; now the wide one is: 8x7B
+// shape, 3072 tokens, up/gate 1630 against 1520 us. It remains as a forced layout.) Shared memory of the narrow layout: four
+// stages and two boxes or three and three, the same times (fine-grained 1000 tokens 323 and 320 us, 256 tokens 147 and 148).
+using BigTile = TileCfg<192, 4, 2, 2, 1, 2, 6>;    // one CTA per SM, two converter groups, two accumulators, two issuers
+using WideTile = TileCfg<192, 2, 1, 1, 2, 1, 3>;      // two CTAs per SM
+using NarrowTile = TileCfg<128, 4, 1, 1, 2, 1, 2>;    // two CTAs per SM, deeper ring
 // (Tried for batches with few tokens per expert and dropped: 64-token tiles with a weight ring of 7 stages instead of
 // 4, and the same tiles with two converter groups per CTA -- 4 groups per SM, 72 registers per thread: Mixtral shape, 64
 // tokens, up/gate 228 and 217 against 226 us; fine-grained 1024 tokens 237 and 239 against 215 us. Neither the weight
@@ -106,11 +113,6 @@ using NarrowTile = TileCfg<128, 4, 1, 1, 2>;    // two CTAs per SM, deeper ring
 // up/gate 489 against 518 us at 768 tokens, 603 against 630 at 1024, 1129 against 1116 at 2048: the third stage is
 // worth 4 - 5 % where the tile count stays the same and loses where 160-token tiles are more tiles; not kept.)
 constexpr int kMaxDownSlices = 4;               // reduction slices of the tensor-core down projection (see plan_down)
-constexpr int kBigMinPerExpert = 640;            // up/gate: ... from which the big layout is used. Re-measured with the exact code conversion (Mixtral
-                                                // shape, us big / wide): 1024 tokens (256 per expert) 695 / 626, 1536 tokens 942 / 873, 2048 tokens 1182 /
-                                                // 1154, 3072 tokens (768 per expert) 1737 / 1785; Mixtral-8x22B shape 1024 tokens 1148 / 991
-constexpr int kWideMinPerExpert = 144;          // up/gate: average routed tokens per expert from which the wide tiles are used (640 tokens
-                                                // over 8 experts: narrow 434, wide 424, big 414 us; 512 tokens: 359 / 380 / 373)
 
 // The B tile is loaded with the smallest box that covers the tile's tokens: boxes of 32, 64, ..., 192 positions.
 constexpr int kBoxStep = 32, kBoxMaps = 6;
@@ -120,6 +122,7 @@ struct TcArgs {
     void* const* slots; const int32_t* slot_map; const Sched* sched;
     const int32_t* count; const int32_t* offset;
     const float* xs_pos; const float* hm_pos; const float* sum_pos; const float* hscale;
+    const CUtensorMap* wmaps;   // [expert][kWeightMaps]
     const int32_t* hexp;        // [2][kMaxExperts]: exponent of the intermediate's magnitude, then the wide-range flag
     __half* h16; __half* h16lo; float* ypart;
     int32_t* status;
@@ -162,11 +165,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     *abort_flag = 1;
     return false;
 }
-__device__ __forceinline__ void cp_async16_s(uint32_t saddr, const void* g) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 
@@ -200,6 +198,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
                    "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
                    "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
                    "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                 : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                  : "r"(taddr) : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
@@ -242,16 +249,16 @@ __device__ __forceinline__ unsigned short f32_to_f16_sat(float v) {
 __device__ __forceinline__ float pow2_f(int e) { return __uint_as_float((unsigned)(max(-126, min(127, e)) + 127) << 23); }
 __device__ __forceinline__ int expo_f(float v) { return (int)((__float_as_uint(v) >> 23) & 0xff) - 127; }
 
-struct Tile { int pos0, ntok, row0, wide, kb0, nkb, split; const unsigned char* blob; };
+struct Tile { int pos0, ntok, row0, wide, kb0, nkb, split, e; const unsigned char* blob; };
 
-// One MMA row's 64 codes of a K-block (shared memory, 64 bytes) -> 32 half2 in k order. SUB: as the fp16
-// subnormals (code + 128) * 2^-24, no subtraction here; else the signed codes, exactly.
+// One MMA row's 64 codes of a K-block (shared memory, 64 bytes, 16-byte pieces exchanged by the XOR of a swizzle) -> 32 half2 in k
+// order. SUB: as the fp16 subnormals (code + 128) * 2^-24, no subtraction here; else the signed codes, exactly.
 template <bool SUB>
-__device__ __forceinline__ void convert_row(unsigned (&f)[32], uint32_t saddr) {
+__device__ __forceinline__ void convert_row(unsigned (&f)[32], uint32_t saddr, uint32_t swizzle) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         unsigned w4[4];
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(w4[0]), "=r"(w4[1]), "=r"(w4[2]), "=r"(w4[3]) : "r"(saddr + q * 16));
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(w4[0]), "=r"(w4[1]), "=r"(w4[2]), "=r"(w4[3]) : "r"((saddr + q * 16) ^ swizzle));
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj) {
             const unsigned u = w4[jj] ^ 0x80808080u;
@@ -266,19 +273,30 @@ __device__ __forceinline__ void convert_row(unsigned (&f)[32], uint32_t saddr) {
     }
 }
 
+// A box of the weights, 128 MMA rows from row0 on x 128 codes from k on (two K-blocks), to shared memory.
+template <bool DOWN> __device__ __forceinline__ void load_weight_box(uint32_t dst, const CUtensorMap* map, int k, int row0, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"((uint32_t)kWBox) : "memory");
+    if (DOWN)
+        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+                     ::"r"(dst), "l"(map), "r"(k), "r"(row0), "r"(bar) : "memory");
+    else
+        asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n"
+                     ::"r"(dst), "l"(map), "r"(k), "r"(0), "r"(row0), "r"(bar) : "memory");
+}
+
 template <bool DOWN, typename TC>
 __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs A, const __grid_constant__ TileMaps bmaps, const __grid_constant__ TileMaps bmaps_lo) {
     constexpr int kTileN = TC::kTileN, kAStages = TC::kStages, kBStages = TC::kStages, kBTileBytes = TC::kBTileBytes;
-    constexpr int kGroups = TC::kGroups, kAccBufs = TC::kAccBufs, kWRing = TC::kWRing;
-    constexpr int kEpiWarp0 = TC::kEpiWarp0, kTmaWarp = TC::kTmaWarp, kMmaWarp = TC::kMmaWarp, kIssuers = TC::kIssuers;
+    constexpr int kGroups = TC::kGroups, kAccBufs = TC::kAccBufs, kWBoxes = TC::kWBoxes;
+    constexpr int kEpiWarp0 = TC::kEpiWarp0, kTmaWarp = TC::kTmaWarp, kMmaWarp = TC::kMmaWarp, kWeightWarp = TC::kWeightWarp, kIssuers = TC::kIssuers;
     constexpr uint32_t kTmemCols = TC::kTmemCols;
     constexpr uint32_t kTmemA = kAccBufs * kTileN;      // first column of the A ring
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_bar[2 * kAStages + 6];   // full, empty, acc_full[2], acc_empty[2], turn[2]
+    __shared__ uint64_t s_bar[2 * kAStages + 6 + 2 * kWBoxes];   // full, empty, acc_full[2], acc_empty[2], turn[2], w_full, w_empty
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     __shared__ int s_ntile[kMaxExperts + 1];          // exclusive prefix of token tiles per active expert
-    __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts];
+    __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts], s_e[kMaxExperts];
     __shared__ int s_wide[kMaxExperts];               // wide-range expert: two fp16 windows of the intermediate (see kLoShift)
     __shared__ const unsigned char* s_blob[kMaxExperts];
     __shared__ int s_nact;
@@ -297,7 +315,7 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     const size_t per = (size_t)R * C;
 
     const uint32_t b_s = smem_u32(smem);                                          // [stage] B tile
-    const uint32_t w_s = b_s + kBStages * kBTileBytes;                            // [group][stage] int8 rows
+    const uint32_t w_s = b_s + kBStages * kBTileBytes;                            // [box] int8 rows
     const uint32_t bar0 = smem_u32(s_bar);
     auto a_full = [&](int s) { return bar0 + 8u * s; };
     auto a_empty = [&](int s) { return bar0 + 8u * (kAStages + s); };
@@ -306,12 +324,15 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     auto acc_full = [&](int b) { return bar0 + 8u * (2 * kAStages + b); };
     auto acc_empty = [&](int b) { return bar0 + 8u * (2 * kAStages + 2 + b); };
     auto turn = [&](int q) { return bar0 + 8u * (2 * kAStages + 4 + q); };
+    auto w_full = [&](int s) { return bar0 + 8u * (2 * kAStages + 6 + s); };
+    auto w_empty = [&](int s) { return bar0 + 8u * (2 * kAStages + 6 + kWBoxes + s); };
 
     // per-expert table: one round of parallel loads, then a serial prefix over shared memory
     const int n_active = A.sched->n_active;
     const bool sub_batch = !DOWN && A.up_conversion == 2;
     if (tid < kMaxExperts && tid < n_active) {
         const int e = A.sched->act_expert[tid];
+        s_e[tid] = e;
         s_cnt[tid] = A.count[e];
         s_off[tid] = A.offset[e];
         s_wide[tid] = A.hexp[kMaxExperts + e];
@@ -320,6 +341,7 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     if (tid == 0) {
         for (int s = 0; s < kAStages; ++s) { mbar_init(a_full(s), 4 + 1); mbar_init(a_empty(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), kIssuers); mbar_init(acc_empty(b), 4); mbar_init(turn(b), 1); }
+        for (int s = 0; s < kWBoxes; ++s) { mbar_init(w_full(s), 1); mbar_init(w_empty(s), 4 * kGroups); }
         s_abort = 0;
         s_nact = n_active;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -373,6 +395,7 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
         t.ntok = min(tn, s_cnt[lo] - nb * tn);
         t.row0 = mb * (DOWN ? kTileM : kTileM / 2);
         t.blob = s_blob[lo];
+        t.e = s_e[lo];
         return t;
     };
     // Ring bookkeeping: K-blocks are numbered over the whole life of the CTA (g = blocks of earlier tiles + kb);
@@ -381,49 +404,32 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     if (warp < kEpiWarp0) {
         // ------------------------------------------------ converters: group (warp >> 2) takes the blocks with g % kGroups == group
         const int group = warp >> 2, gw = warp & 3, row = gw * 32 + lane;     // MMA row of this thread
-        const uint32_t w_g = w_s + group * (kWRing * kWStage) + gw * kWWarp;
-        const uint32_t w_cp = w_g + (lane & 7) * kWRow + (lane >> 3) * 16;   // + stage * kWStage + i * 8 * kWRow
-        const uint32_t w_rd = w_g + lane * kWRow;                             // + stage * kWStage + q * 16
+        const uint32_t w_rd = w_s + row * 128, swizzle = (uint32_t)(row & 7) << 4;
         uint32_t gbase = 0;                                                   // K-blocks of this CTA's earlier tiles
+        int ws = 0;                                                           // box of the weight ring and the parity of its 'full' barrier
+        uint32_t wp = 0;
         for (long tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x) {
             const Tile t = decode(tile);
             const int nkb = t.nkb;                              // K-blocks of this tile (a slice of the reduction in S5)
             const bool sub = sub_batch && !t.wide;              // offset subnormals or exact codes: per tile, see above
-            // source of the row this lane copies in instruction 0 (MMA row 32 gw + (lane & 7)); instruction i is 8 MMA
-            // rows further: + 8 rows of W2^ (S5) or + 4 expert-hidden rows of W1^ / W3^ (S4)
-            const unsigned char* src;
-            size_t src_step;
-            {
-                const int mrow = gw * 32 + (lane & 7);
-                if (DOWN) { src = t.blob + per + (size_t)(t.row0 + mrow) * R + (lane >> 3) * 16 + (size_t)t.kb0 * kKB; src_step = (size_t)8 * R; }
-                else { src = t.blob + ((mrow & 1) ? 2 * per : 0) + (size_t)(t.row0 + (mrow >> 1)) * C + (lane >> 3) * 16; src_step = (size_t)4 * C; }
-            }
             const int kb0 = (int)(((uint32_t)group + kGroups - gbase % kGroups) % kGroups);   // first K-block of this tile that belongs to the group
-            const int nmine = (nkb - kb0 + kGroups - 1) / kGroups;                               // its blocks: kb0, kb0 + kGroups, ...
-#pragma unroll
-            for (int s = 0; s < kWRing - 1; ++s) {
-                if (s < nmine) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cp_async16_s(w_cp + s * kWStage + i * 8 * kWRow, src + i * src_step + (size_t)(kb0 + kGroups * s) * kKB);
-                }
-                cp_async_commit();
-            }
             bool ok = true;
-            for (int j = 0; j < nmine; ++j) {
-                const int pre = j + kWRing - 1;
-                if (pre < nmine) {
-                    const int ws = pre % kWRing;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cp_async16_s(w_cp + ws * kWStage + i * 8 * kWRow, src + i * src_step + (size_t)(kb0 + kGroups * pre) * kKB);
+            for (int kb = 0; kb < nkb; ++kb) {                  // box kb / 2; every warp waits for every box and hands it back
+                if ((kb & 1) == 0 && !mbar_wait(w_full(ws), wp, &s_abort, A.spin_limit)) { ok = false; break; }
+                const bool mine = kGroups == 1 || kb % kGroups == kb0;
+                unsigned f[32];                                 // 64 codes as fp16, in k order
+                if (mine) {
+                    const uint32_t at = w_rd + ws * kWBox + (kb & 1) * 64;
+                    if (sub) convert_row<true>(f, at, swizzle);
+                    else convert_row<false>(f, at, swizzle);
                 }
-                cp_async_commit();
-                cp_async_wait<kWRing - 1>();
-                __syncwarp();                                     // the other lanes' copies of this stage have landed too
-                const int ws = j % kWRing;
-                unsigned f[32];                                   // 64 codes as fp16, in k order
-                if (sub) convert_row<true>(f, w_rd + ws * kWStage);
-                else convert_row<false>(f, w_rd + ws * kWStage);
-                const uint32_t g = gbase + (uint32_t)(kb0 + kGroups * j);
+                if ((kb & 1) || kb + 1 == nkb) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(w_empty(ws));
+                    if (++ws == kWBoxes) { ws = 0; wp ^= 1u; }
+                }
+                if (!mine) continue;
+                const uint32_t g = gbase + (uint32_t)kb;
                 const uint32_t st = g % kAStages;
                 if (!mbar_wait(a_empty(st), ((g / kAStages) & 1u) ^ 1u, &s_abort, A.spin_limit)) { ok = false; break; }
                 tc_fence_after();
@@ -433,8 +439,6 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(a_full(st));
             }
-            cp_async_wait<0>();
-            (void)row;
             if (!ok) break;
             gbase += (uint32_t)nkb;
         }
@@ -457,20 +461,20 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
                 float* yp = A.ypart + (size_t)t.split * A.ypart_stride;
                 auto store = [&](auto wide_c) {       // compiled with and without the second window, chosen per tile
                     constexpr bool kWide = decltype(wide_c)::value;
-                    for (int c0 = 0; c0 < ncol; c0 += 32) {
-                        uint32_t v[32];
+                    for (int c0 = 0; c0 < ncol; c0 += 16) {
+                        uint32_t v[16];
                         __syncwarp();
-                        tmem_ld32(acc_t + c0, v);
+                        tmem_ld16(acc_t + c0, v);
                         if (kWide) {                  // the lower window's sums sit one box further, scaled by 2^kLoShift
-                            uint32_t w[32];
+                            uint32_t w[16];
                             __syncwarp();
-                            tmem_ld32(acc_t + ncol + c0, w);
+                            tmem_ld16(acc_t + ncol + c0, w);
                             const float lo_scale = pow2_f(-kLoShift);
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaf(__uint_as_float(w[j]), lo_scale, __uint_as_float(v[j])));
+                            for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(fmaf(__uint_as_float(w[j]), lo_scale, __uint_as_float(v[j])));
                         }
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
+                        for (int j = 0; j < 16; ++j) {
                             const int n = c0 + j;
                             if (n < t.ntok) yp[(size_t)(t.pos0 + n) * C + c] = __uint_as_float(v[j]) * (__ldg(A.hscale + t.pos0 + n) * so);
                         }
@@ -490,12 +494,12 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
                 // the form is chosen per tile, so that no per-element branch sits in it.
                 auto finish = [&](auto sub_c, auto wide_c) {
                     constexpr bool kSub = decltype(sub_c)::value, kWide = decltype(wide_c)::value;
-                    for (int c0 = 0; c0 < ncol; c0 += 32) {
-                        uint32_t v[32];
+                    for (int c0 = 0; c0 < ncol; c0 += 16) {
+                        uint32_t v[16];
                         __syncwarp();
-                        tmem_ld32(acc_t + c0, v);
+                        tmem_ld16(acc_t + c0, v);
 #pragma unroll
-                        for (int jj = 0; jj < 16; ++jj) {
+                        for (int jj = 0; jj < 8; ++jj) {
                             const float a = __uint_as_float(v[2 * jj]), b = __uint_as_float(v[2 * jj + 1]);
                             // one exchange per pair: the even lane needs its neighbour's G of the even column, the odd lane
                             // its neighbour's U of the odd column
@@ -564,6 +568,27 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
                 if (!ok) break;
             }
         }
+    } else if (warp == kWeightWarp) {
+        // ------------------------------------------------ weight producer: one lane, one TMA load per box of two K-blocks (the last
+        // one of an odd number of K-blocks holds one that nobody reads). The maps were made by the routing kernels.
+        if (lane == 0) {
+            int ws = 0;
+            uint32_t wp = 1;
+            const CUtensorMap* last_map = nullptr;
+            for (long tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x) {
+                const Tile t = decode(tile);
+                const CUtensorMap* map = A.wmaps + (size_t)t.e * kWeightMaps + (DOWN ? 7 : 3);
+                if (map != last_map) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(map) : "memory");
+                last_map = map;
+                bool ok = true;
+                for (int kb = 0; kb < t.nkb; kb += 2) {
+                    if (!mbar_wait(w_empty(ws), wp, &s_abort, A.spin_limit)) { ok = false; break; }
+                    load_weight_box<DOWN>(w_s + ws * kWBox, map, (t.kb0 + kb) * kKB, t.row0, w_full(ws));
+                    if (++ws == kWBoxes) { ws = 0; wp ^= 1u; }
+                }
+                if (!ok) break;
+            }
+        }
     } else {
         // ------------------------------------------------ MMA issuers (one lane each). With two, issuer q takes the
         // K-blocks with running index g = q (mod 2); before its MMAs it waits for the other issuer's turn signal, so
@@ -615,7 +640,10 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     // ---------------------------------------------------- common exit
     tc_fence_before();
     __syncthreads();
-    if (s_abort && tid == 0) atomicOr(A.status, 2);      // after the barrier: the role that gave up may be the last to arrive
+    if (s_abort) {                       // after the barrier: the role that gave up may be the last to arrive
+        if (tid == 0) atomicOr(A.status, 2);
+        for (int i = 0; i < 50; ++i) __nanosleep(1000);      // copies in flight land within microseconds
+    }
     if (warp == kTmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
@@ -647,7 +675,9 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
 constexpr int kPairGroups = 2, kPairAcc = 2;
 constexpr int kPairEpiWarp0 = 4 * kPairGroups, kPairTmaWarp = kPairEpiWarp0 + 4, kPairMmaWarp = kPairEpiWarp0 + 5;
 constexpr int kPairIssuers = 2;                       // MMA-issuing warps of the leader, taking the K-blocks in turn
-constexpr int kPairThreads = (kPairMmaWarp + kPairIssuers) * 32;
+constexpr int kPairWeightWarp = kPairMmaWarp + kPairIssuers;
+constexpr int kPairThreads = (kPairWeightWarp + 1) * 32;
+constexpr int kPairWBoxes = 6;                        // weight ring, boxes of two K-blocks
 constexpr uint32_t kPairTmemCols = 512;
 constexpr int kHalfBoxStep = 16, kHalfBoxMaps = 6;                    // half-tile boxes of 16, 32, ..., 96 positions
 // TN tokens per tile, NS ring stages (A ring in TMEM, B ring in shared memory): two accumulators of TN columns and
@@ -656,7 +686,7 @@ template <int TN, int NS> struct PairCfg {
     static constexpr int kTileN = TN, kStages = NS;
     static constexpr uint32_t kTmemA = kPairAcc * TN;
     static constexpr int kBHalfBytes = (TN / 2) * kKB * 2;           // one CTA's half of the activation tile, per stage
-    static constexpr size_t kSmem = (size_t)NS * kBHalfBytes + (size_t)kPairGroups * kWStages * kWStage + 1024;
+    static constexpr size_t kSmem = (size_t)NS * kBHalfBytes + (size_t)kPairWBoxes * kWBox + 1024;
     static_assert(kTmemA + NS * 32 <= kPairTmemCols, "TMEM columns");
     static_assert(TN / 2 <= kHalfBoxStep * kHalfBoxMaps && TN % 64 == 0, "boxes cover a half tile");
 };
@@ -700,11 +730,11 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
     constexpr int kPairTileN = PC::kTileN, kPairStages = PC::kStages, kPairBHalfBytes = PC::kBHalfBytes;
     constexpr uint32_t kPairTmemA = PC::kTmemA;
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_bar[2 * kPairStages + 6];   // full, empty, acc_full[2], acc_empty[2], turn[2]
+    __shared__ uint64_t s_bar[2 * kPairStages + 6 + 2 * kPairWBoxes];   // full, empty, acc_full[2], acc_empty[2], turn[2], w_full, w_empty
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     __shared__ int s_ntile[kMaxExperts + 1];
-    __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts], s_wide[kMaxExperts];
+    __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts], s_wide[kMaxExperts], s_e[kMaxExperts];
     __shared__ const unsigned char* s_blob[kMaxExperts];
     __shared__ int s_nact;
 
@@ -724,11 +754,14 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
     auto acc_full = [&](int b) { return bar0 + 8u * (2 * kPairStages + b); };
     auto acc_empty = [&](int b) { return bar0 + 8u * (2 * kPairStages + 2 + b); };
     auto turn = [&](int q) { return bar0 + 8u * (2 * kPairStages + 4 + q); };
+    auto w_full = [&](int s) { return bar0 + 8u * (2 * kPairStages + 6 + s); };
+    auto w_empty = [&](int s) { return bar0 + 8u * (2 * kPairStages + 6 + kPairWBoxes + s); };
 
     const int n_active = A.sched->n_active;
     const bool sub_batch = !DOWN && A.up_conversion == 2;
     if (tid < kMaxExperts && tid < n_active) {
         const int e = A.sched->act_expert[tid];
+        s_e[tid] = e;
         s_cnt[tid] = A.count[e];
         s_off[tid] = A.offset[e];
         s_wide[tid] = A.hexp[kMaxExperts + e];
@@ -737,6 +770,7 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
     if (tid == 0) {
         for (int s = 0; s < kPairStages; ++s) { mbar_init(full(s), 4 + 4 + 1); mbar_init(empty(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), kPairIssuers); mbar_init(acc_empty(b), 4 + 4); mbar_init(turn(b), 1); }
+        for (int s = 0; s < kPairWBoxes; ++s) { mbar_init(w_full(s), 1); mbar_init(w_empty(s), 4 * kPairGroups); }
         s_abort = 0;
         s_nact = n_active;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -777,6 +811,7 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
         t.ntok = min(tn, s_cnt[lo] - nb * tn);
         t.row0 = mb * (DOWN ? 2 * kTileM : kTileM) + (int)rank * (DOWN ? kTileM : kTileM / 2);   // this CTA's first row
         t.blob = s_blob[lo];
+        t.e = s_e[lo];
         return t;
     };
     // Columns of the pair's MMA and what each CTA loads for them. Ordinary tile: N = the tokens rounded up to 32, the
@@ -788,47 +823,32 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
 
     if (warp < kPairEpiWarp0) {
         // ------------------------------------------------ converters (as in the one-CTA kernel; the 'full' arrival goes to the leader)
-        const int group = warp >> 2, gw = warp & 3;
-        const uint32_t w_g = w_s + group * (kWStages * kWStage) + gw * kWWarp;
-        const uint32_t w_cp = w_g + (lane & 7) * kWRow + (lane >> 3) * 16;
-        const uint32_t w_rd = w_g + lane * kWRow;
+        const int group = warp >> 2, gw = warp & 3, row = gw * 32 + lane;
+        const uint32_t w_rd = w_s + row * 128, swizzle = (uint32_t)(row & 7) << 4;
         uint32_t gbase = 0;
+        int ws = 0;
+        uint32_t wp = 0;
         for (long tile = pair_id; tile < total && !s_abort; tile += n_pairs, gbase += (uint32_t)nkb) {
             const Tile t = decode(tile);
             const bool sub = sub_batch && !t.wide;
-            const unsigned char* src;
-            size_t src_step;
-            {
-                const int mrow = gw * 32 + (lane & 7);
-                if (DOWN) { src = t.blob + per + (size_t)(t.row0 + mrow) * R + (lane >> 3) * 16; src_step = (size_t)8 * R; }
-                else { src = t.blob + ((mrow & 1) ? 2 * per : 0) + (size_t)(t.row0 + (mrow >> 1)) * C + (lane >> 3) * 16; src_step = (size_t)4 * C; }
-            }
             const int kb0 = (int)(((uint32_t)group + kPairGroups - gbase % kPairGroups) % kPairGroups);
-            const int nmine = (nkb - kb0 + kPairGroups - 1) / kPairGroups;
-#pragma unroll
-            for (int s = 0; s < kWStages - 1; ++s) {
-                if (s < nmine) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cp_async16_s(w_cp + s * kWStage + i * 8 * kWRow, src + i * src_step + (size_t)(kb0 + kPairGroups * s) * kKB);
-                }
-                cp_async_commit();
-            }
             bool ok = true;
-            for (int j = 0; j < nmine; ++j) {
-                const int pre = j + kWStages - 1;
-                if (pre < nmine) {
-                    const int ws = pre % kWStages;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cp_async16_s(w_cp + ws * kWStage + i * 8 * kWRow, src + i * src_step + (size_t)(kb0 + kPairGroups * pre) * kKB);
-                }
-                cp_async_commit();
-                cp_async_wait<kWStages - 1>();
-                __syncwarp();
-                const int ws = j % kWStages;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if ((kb & 1) == 0 && !mbar_wait(w_full(ws), wp, &s_abort, A.spin_limit)) { ok = false; break; }
+                const bool mine = kb % kPairGroups == kb0;
                 unsigned f[32];
-                if (sub) convert_row<true>(f, w_rd + ws * kWStage);
-                else convert_row<false>(f, w_rd + ws * kWStage);
-                const uint32_t g = gbase + (uint32_t)(kb0 + kPairGroups * j);
+                if (mine) {
+                    const uint32_t at = w_rd + ws * kWBox + (kb & 1) * 64;
+                    if (sub) convert_row<true>(f, at, swizzle);
+                    else convert_row<false>(f, at, swizzle);
+                }
+                if ((kb & 1) || kb + 1 == nkb) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(w_empty(ws));
+                    if (++ws == kPairWBoxes) { ws = 0; wp ^= 1u; }
+                }
+                if (!mine) continue;
+                const uint32_t g = gbase + (uint32_t)kb;
                 const uint32_t st = g % kPairStages;
                 if (!mbar_wait(empty(st), ((g / kPairStages) & 1u) ^ 1u, &s_abort, A.spin_limit)) { ok = false; break; }
                 tc_fence_after();
@@ -838,7 +858,6 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(map_to_cta(full(st), 0));
             }
-            cp_async_wait<0>();
             if (!ok) break;
         }
     } else if (warp < kPairTmaWarp) {
@@ -929,6 +948,26 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty(buf), 0));
         }
+    } else if (warp == kPairWeightWarp) {
+        // ------------------------------------------------ weight producer of this CTA's rows (as in the one-CTA kernel)
+        if (lane == 0) {
+            int ws = 0;
+            uint32_t wp = 1;
+            const CUtensorMap* last_map = nullptr;
+            for (long tile = pair_id; tile < total && !s_abort; tile += n_pairs) {
+                const Tile t = decode(tile);
+                const CUtensorMap* map = A.wmaps + (size_t)t.e * kWeightMaps + (DOWN ? 7 : 3);
+                if (map != last_map) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(map) : "memory");
+                last_map = map;
+                bool ok = true;
+                for (int kb = 0; kb < nkb; kb += 2) {
+                    if (!mbar_wait(w_empty(ws), wp, &s_abort, A.spin_limit)) { ok = false; break; }
+                    load_weight_box<DOWN>(w_s + ws * kWBox, map, kb * kKB, t.row0, w_full(ws));
+                    if (++ws == kPairWBoxes) { ws = 0; wp ^= 1u; }
+                }
+                if (!ok) break;
+            }
+        }
     } else if (warp == kPairTmaWarp) {
         // ------------------------------------------------ this CTA's half of the activation tile, one load per K-block
         if (lane == 0) {
@@ -1004,7 +1043,10 @@ k_ffn_tc_pair(TcArgs A, const __grid_constant__ HalfMaps bmaps, const __grid_con
     // ---------------------------------------------------- common exit
     tc_fence_before();
     __syncthreads();
-    if (s_abort && tid == 0) atomicOr(A.status, 2);
+    if (s_abort) {
+        if (tid == 0) atomicOr(A.status, 2);
+        for (int i = 0; i < 50; ++i) __nanosleep(1000);      // copies in flight land within microseconds
+    }
     cluster_sync_all();                                // the peer's tensor and shared memory are no longer in use by this CTA
     if (warp == kPairTmaWarp) {
         tc_fence_after();
@@ -1064,6 +1106,7 @@ TcArgs make_tc_args(mira_ctx* ctx, void* const* slots, const int32_t* slot_map) 
     TcArgs A;
     A.slots = slots; A.slot_map = slot_map;
     A.sched = ws_ptr<Sched>(ctx, ctx->lay.sched);
+    A.wmaps = ws_ptr<CUtensorMap>(ctx, ctx->lay.wmaps);
     A.count = ws_ptr<int32_t>(ctx, ctx->lay.count);
     A.offset = ws_ptr<int32_t>(ctx, ctx->lay.offset);
     A.xs_pos = ws_ptr<float>(ctx, ctx->lay.xs_pos);
@@ -1126,15 +1169,19 @@ static void launch_cfg(mira_ctx* ctx, const TcArgs& A, const unsigned char (*map
     launch_pdl(k_ffn_tc<DOWN, TC>, dim3(ctx->n_sm * TC::kCtasPerSm), dim3(TC::kThreads), TC::kSmem, st, A, tm, tm_lo);
 }
 
+// Token tiles of a step with tiles of `tn` tokens: exact for the shared experts, tokens / tn plus half a ragged tile per expert for the
+// routed ones (at least one per expert that can be routed to).
+static double token_tiles(const mira_ctx* ctx, int tn) {
+    const double T = ctx->route_T, E = ctx->cfg.n_experts, pairs = T * ctx->route_k;
+    return std::max(std::min(E, pairs), pairs / tn + 0.5 * std::min(E, pairs)) + ctx->cfg.n_shared * std::ceil(T / tn);
+}
 // Estimated cost of a down projection in a 2-CTA layout with tiles of `tn` tokens: the kernel has few row tiles
 // (C / 128), so what counts is how many ROUNDS of tiles its CTAs run, times the cost of a tile relative to a narrow
-// one (a wide tile covers 1.5 times the tokens at 1.3 times the time: 224 K-blocks take 115 us narrow, 150 us wide).
-// Token-tile columns: exact for the shared experts, tokens / tn plus half a ragged tile per expert for the routed ones
-// (at least one per expert that can be routed to).
+// one (a wide tile covers 1.5 times the tokens at kWideCostDown times the time: whole rounds of the 8x7B shape, 2048 tokens, four narrow
+// 530 us, three wide 500).
+constexpr double kWideCostDown = 1.25;
 static double down_cost(const mira_ctx* ctx, int tn, double tile_cost, int slices = 1) {
-    const double T = ctx->route_T, E = ctx->cfg.n_experts, pairs = T * ctx->route_k;
-    const double cols = std::max(std::min(E, pairs), pairs / tn + 0.5 * std::min(E, pairs)) + ctx->cfg.n_shared * std::ceil(T / tn);
-    const double tiles = cols * (ctx->cfg.hidden / kTileM) * slices;
+    const double tiles = token_tiles(ctx, tn) * (ctx->cfg.hidden / kTileM) * slices;
     return std::ceil(tiles / (2.0 * ctx->n_sm)) * tile_cost;
 }
 
@@ -1165,10 +1212,9 @@ static DownPlan plan_down(const mira_ctx* ctx) {
     p.splits = 1;
     const bool narrow_only = 2 * avg < NarrowTile::kTileN;
     if (p.layout == 0)
-        // wide only when the estimate is clearly lower: near a tie the narrow layout is the safer one (1536 tokens: 429 / 460)
         // (with fewer than half a narrow tile of tokens per expert on average no expert fills a wide tile: narrow.
         // Fine-grained layer, 128 tokens: 39 against 45 us)
-        p.layout = (narrow_only || 0.9 * down_cost(ctx, NarrowTile::kTileN, 1.0) <= down_cost(ctx, WideTile::kTileN, 1.3)) ? 1 : 2;
+        p.layout = (narrow_only || down_cost(ctx, NarrowTile::kTileN, 1.0) <= down_cost(ctx, WideTile::kTileN, kWideCostDown)) ? 1 : 2;
     if ((p.layout == 4 || p.layout == 5) && !pair_shape_ok(ctx->cfg)) p.layout = 2;
     if (p.layout >= 4) return p;                           // the two-SM kernel takes whole reductions
     const int nkb = ctx->cfg.ffn / kKB;
@@ -1176,11 +1222,11 @@ static DownPlan plan_down(const mira_ctx* ctx) {
     if (ctx->down_slices_forced > 0) { p.splits = std::min(ctx->down_slices_forced, std::min(ctx->down_splits, nkb)); return p; }
     if (ctx->tc_layout != 0) return p;                     // a forced layout keeps whole reductions unless slices are forced too
     auto cost = [&](int tn, double w, int S) { return down_cost(ctx, tn, 1.0, S) * (w * nkb / S + 26.0); };
-    const double w0 = p.layout == 1 ? 1.0 : 1.3;
+    const double w0 = p.layout == 1 ? 1.0 : kWideCostDown;
     double best = cost(p.layout == 1 ? NarrowTile::kTileN : WideTile::kTileN, w0, 1);
     for (int S = 2; S <= max_s; ++S)
         for (int lay = 1; lay <= (narrow_only ? 1 : 2); ++lay) {
-            const double c = cost(lay == 1 ? NarrowTile::kTileN : WideTile::kTileN, lay == 1 ? 1.0 : 1.3, S);
+            const double c = cost(lay == 1 ? NarrowTile::kTileN : WideTile::kTileN, lay == 1 ? 1.0 : kWideCostDown, S);
             if (c < 0.93 * best) { best = c; p.layout = lay; p.splits = S; }     // slices cost partial-sum traffic: only for a clear gain
         }
     return p;
@@ -1190,15 +1236,16 @@ int down_tc_slices(const mira_ctx* ctx) { return plan_down(ctx).splits; }
 
 template <bool DOWN>
 static void launch_tc(mira_ctx* ctx, TcArgs& A, const unsigned char (*maps)[128], cudaStream_t st) {
-    // Up/gate has many row tiles (R / 64), so its time follows the number of tiles: narrow tiles while an expert gets
-    // fewer tokens than fill wide ones on average, then wide, and with few experts and many tokens the big layout.
-    // The down projection is chosen by the estimated number of rounds (measured on the Mixtral shape, us narrow /
-    // wide: 384 tokens 186 / 160, 896 tokens 229 / 300, 1024 tokens 311 / 291, 3072 tokens 730 / 664: the estimate
-    // picks the faster one in each case).
-    const long avg = (long)ctx->route_T * ctx->route_k / (ctx->cfg.n_experts > 0 ? ctx->cfg.n_experts : 1);
+    // Up/gate has many row tiles (R / 64), so its time follows the number of tiles; a wide tile of the same tokens takes about 1.1
+    // times a narrow one's. Measured, us narrow / wide: 8x7B shape, 300 tokens 250 / 271, 450: 351 / 348, 700: 468 / 426, 2048: 1222 /
+    // 1029; 8x22B shape, 300 tokens 451 / 470; fine-grained layer 256 tokens 83 / 94, 600: 135 / 139, 1000 (half of the pairs in
+    // the shared experts) 187 / 177, 2000: 307 / 286; hidden 2304, ffn 2816, 16 experts, one shared, 600 tokens 112 / 108.
+    // The down projection is chosen by the estimated number of rounds: 8x7B shape 700 tokens 245 / 293, 900: 268 / 302, 1200: 360 /
+    // 330, 1536: 477 / 475, 2048: 530 / 500, 3072: 774 / 702; 8x22B shape 300 tokens 262 / 330, 700: 423 / 389; fine-grained layer 600
+    // tokens 73 / 81, 1000: 99 / 104, 2000: 155 / 150: the estimate picks the faster one in each case.
     int layout = ctx->tc_layout;                          // 0 unless a layout is forced (MIRA_OPT_TENSOR_LAYOUT)
     if (layout == 0 && !DOWN) {
-        layout = avg < kWideMinPerExpert ? 1 : (avg >= kBigMinPerExpert && ctx->cfg.n_experts <= 16) ? 3 : 2;
+        layout = 1.1 * token_tiles(ctx, WideTile::kTileN) < token_tiles(ctx, NarrowTile::kTileN) ? 2 : 1;
     }
     if (DOWN) { const DownPlan p = plan_down(ctx); layout = p.layout; A.down_splits = p.splits; }
     if ((layout == 4 || layout == 5) && !pair_shape_ok(ctx->cfg)) layout = DOWN ? 2 : 3;
