@@ -60,17 +60,24 @@ __device__ __forceinline__ void warp_topk(float (&v)[8], int E, int k, int lane,
     else warp_topk_n<8>(v, E, k, lane, out_idx, out_val);
 }
 
-// The same selection with the results spread over the lanes: lane j (< k) returns the j-th selection. Used by the
-// single-CTA routing kernel (at most 16 experts: one slot per lane).
-__device__ __forceinline__ void warp_topk_lanes(float (&v)[8], int E, int k, int lane, int& my_idx, float& my_val) {
+// The same selection with the results spread over the lanes: lane j (< k) returns the j-th selection of the E scores at v.
+template <int SLOTS>
+__device__ __forceinline__ void warp_topk_lanes_n(const float* v, int E, int k, int lane, int& my_idx, float& my_val) {
     my_idx = 0; my_val = -INFINITY;
-    unsigned key[1] = {lane < E ? topk_key(v[0]) : 0u};
+    unsigned key[SLOTS];
+#pragma unroll
+    for (int i = 0; i < SLOTS; ++i) key[i] = lane + 32 * i < E ? topk_key(v[lane + 32 * i]) : 0u;
 #pragma unroll 1
     for (int j = 0; j < k; ++j) {
         int bi; unsigned bk;
-        topk_step<1>(key, lane, bi, bk);
+        topk_step<SLOTS>(key, lane, bi, bk);
         if (lane == j) { my_idx = bi; my_val = topk_value(bk); }
     }
+}
+__device__ __forceinline__ void warp_topk_lanes(const float* v, int E, int k, int lane, int& my_idx, float& my_val) {
+    if (E <= 32) warp_topk_lanes_n<1>(v, E, k, lane, my_idx, my_val);
+    else if (E <= 64) warp_topk_lanes_n<2>(v, E, k, lane, my_idx, my_val);
+    else warp_topk_lanes_n<8>(v, E, k, lane, my_idx, my_val);
 }
 
 // Routing weight of lane j's selection: softmax over the k selected logits, the sum taken in selection order
@@ -699,191 +706,209 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
     if (threadIdx.x == 0) *A.ticket = 0u;
 }
 
-// Fused S1-S3 (+ schedule) for decode-sized batches in ONE CTA: no ticket, no fences, no atomics on the
-// common path. Requires T * C * 2 bytes of shared memory for the token rows (T <= kSingleCtaMaxTokens).
-constexpr int kSingleCtaMaxTokens = 4;      // beyond, one CTA per token is faster (8 tokens x 8 experts: 23 against 18 us)
-constexpr int kSingleCtaThreads = 512;
+// Fused S1-S3 (+ schedule) for the smallest batches: a chain of latencies that HBM idles through, in one cluster of 8 CTAs. CTA q
+// scores the experts q, q + 8, ... for all tokens; the scores meet in CTA 0 through distributed shared memory (one cluster barrier;
+// no ticket, no fences), which selects, groups and writes the schedule while the others write the fp16 copies of the tokens.
+// Every score is one warp's sum in the order that the other routing kernels use, so all give the same bits.
+// What bounds it: round trips, and code that is run once per step and fetched cold (from L2 at best): the loops stay rolled and
+// the tail has as few instructions and barriers as it can. Measured, us per step, before (up to 16 experts in one CTA, else a CTA
+// per token and a ticket) -> now: 8x7B shape, 1 token 71.2 -> 69.9, 4: 133.9 -> 130.6; fine-grained layer, 1 token 34.8 -> 30.1, 4: 39.3
+// -> 35.9; 1024 x 512, 16 experts, 4 tokens 24.2 -> 20.0; 200 experts, 2 tokens 40.7 -> 29.8. From the previous step's end on, 8x7B /
+// fine-grained with 4 tokens: rows staged 1.4 / 1.0, scores 3.2 / 3.8, cluster barrier 3.7 / 4.5, selection 4.0 / 5.3, all written 5.3 / 6.8
+// us. Tried: the scores' loops unrolled over the tokens (decode of 8x7B 72.2); warps that run the tail's code once ahead of time
+// (39.2 against 37.2 then: they fetch the same lines from the same place).
+constexpr int kClusterCtas = 8, kClusterThreads = 512, kClusterMaxTokens = 4;
 
-__global__ void __launch_bounds__(kSingleCtaThreads) k_route_small(TokenArgs A, GroupArgs G, SchedArgs S) {
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads) k_route_cluster(const __grid_constant__ TokenArgs A, const __grid_constant__ GroupArgs G, const __grid_constant__ SchedArgs S) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint4* xs = reinterpret_cast<uint4*>(smem);                        // [T][C/8]
-    __shared__ float s_sc[kSingleCtaMaxTokens][kMaxExperts];
-    __shared__ int s_idx[kSingleCtaMaxTokens][kMaxTopK];
-    __shared__ int s_rank[kSingleCtaMaxTokens][kMaxTopK];
-    __shared__ int s_count[kMaxExperts];
-    __shared__ int s_off[kMaxExperts + 1];
+    __shared__ float s_sc[kClusterMaxTokens][kMaxExperts];             // CTA 0: the scores
+    __shared__ float s_red[3][32];
+    __shared__ int s_idx[kClusterMaxTokens * kMaxTopK];
     __shared__ unsigned s_word[kMaxExperts / 32];
     __shared__ int s_slot[kMaxExperts];
     const int T = A.T, C = A.C, E = A.E, k = A.k, c8 = C / 8, ns = G.ns, Etot = E + ns, kk = k + ns;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = kSingleCtaThreads / 32;
-    if ((int)blockIdx.x >= S.n_main) {       // statistics CTAs: one per expert, beside the routing CTA
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = blockIdx.x;
+    constexpr int kWarps = kClusterThreads / 32;
+    if (q >= S.n_main) {       // statistics and prefetch CTAs beside the routing cluster
         pdl_wait();
         pdl_launch();
-        if ((int)blockIdx.x < S.n_main + S.n_stat) expert_stats(S, blockIdx.x - S.n_main);
-        else prefetch_shared(S, E, ns, blockIdx.x - S.n_main - S.n_stat);
+        if (q < S.n_main + S.n_stat) expert_stats(S, q - S.n_main);
+        else if (q < S.n_main + S.n_stat + S.n_pre) prefetch_shared(S, E, ns, q - S.n_main - S.n_stat);
         return;
     }
-    prefetch_rows_l2(A.W, C * 2, warp, nwarps, E, lane);     // the router is constant: ask for it under the previous kernel's tail
+    // Experts of this CTA (local number le: expert q + 8 le); g warps share an expert, each takes every g-th token.
+    const int n_own = (E - q + kClusterCtas - 1) / kClusterCtas;
+    const int g = max(1, min(T, kWarps / max(1, n_own))), slots = kWarps / g, first = warp / g, tq = warp % g;
+    const bool scores = warp < slots * g;
+    for (int le = first; scores && le < n_own; le += slots)            // the router is constant: ask for it under the previous kernel's tail
+        if (tq == 0) prefetch_rows_l2(A.W, C * 2, q + kClusterCtas * le, E, q + kClusterCtas * le + 1, lane);
     pdl_wait();            // the previous step's kernels still read the buffers this kernel rewrites
     pdl_launch();
-    // Every load that does not depend on another is issued before the first barrier, so a cold L2 costs
-    // one DRAM round trip, not one per step: token rows, residency of every expert, bias, and the
-    // first batch of this warp's router rows.
+    // Every load that does not depend on another is issued before the first barrier.
     const uint4* xg = reinterpret_cast<const uint4*>(A.x);
-    for (int i = threadIdx.x; i < T * c8; i += kSingleCtaThreads) xs[i] = xg[i];
-    if (A.do_sched) for (int e = threadIdx.x; e < Etot; e += kSingleCtaThreads) s_slot[e] = S.slot_map[e];
+    for (int i = threadIdx.x; i < T * c8; i += kClusterThreads) xs[i] = xg[i];
     const uint4* wg = reinterpret_cast<const uint4*>(A.W);
     constexpr int kWB = 16;                                  // router chunks per lane held in registers
     uint4 wpre[kWB];
-    {
-        const int e = warp;                                  // first expert of this warp
+    auto fetch = [&](int le, int i0) {
+        const int e = q + kClusterCtas * le;
 #pragma unroll
         for (int j = 0; j < kWB; ++j) {
-            const int i = lane + 32 * j;
-            wpre[j] = (e < E && i < c8) ? __ldg(wg + (size_t)e * c8 + i) : make_uint4(0, 0, 0, 0);
+            const int i = i0 + lane + 32 * j;
+            if (i0 + 32 * j >= c8) break;
+            wpre[j] = (scores && le < n_own && i < c8) ? __ldg(wg + (size_t)e * c8 + i) : make_uint4(0, 0, 0, 0);
         }
+    };
+    fetch(first, 0);
+    if (q == 0 && A.do_sched) {
+        for (int e = threadIdx.x; e < Etot; e += kClusterThreads) s_slot[e] = S.slot_map[e];
     }
-    const float bpre = (A.bias && warp < E) ? A.bias[warp] : 0.f;
     __syncthreads();
-    // per token (one warp each, from the last warp down: the first warps have a router row to score): power-of-two
-    // fp16 scale, norm, sum, fp16 copy
-    for (int t = nwarps - 1 - warp; t < T; t += nwarps) {
-        float m = 0.f;
-        for (int i = lane; i < c8; i += 32) {
-            const uint4 v = xs[t * c8 + i];
-            const unsigned w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) m = fmaxf(m, fmaxf(fabsf(bf16lo(w4[j])), fabsf(bf16hi(w4[j]))));
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        int ex = expo_of(m);
-        ex = (m > 0.f) ? max(-100, min(127, ex)) : 13;
-        const float sc_up = __uint_as_float((unsigned)(127 + 13 - ex) << 23);
-        const float sc_dn = __uint_as_float((unsigned)(127 - 13 + ex) << 23);
-        float ss = 0.f, sm = 0.f;
-        uint4* og = reinterpret_cast<uint4*>(A.x16) + (size_t)t * c8;
-        for (int i = lane; i < c8; i += 32) {
-            const uint4 v = xs[t * c8 + i];
-            const unsigned w4[4] = {v.x, v.y, v.z, v.w};
-            unsigned o4[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float a = bf16lo(w4[j]) * sc_up, b = bf16hi(w4[j]) * sc_up;
-                ss = fmaf(a, a, ss); ss = fmaf(b, b, ss);
-                const __half2 h = __floats2half2_rn(a, b);
-                const float2 hf = __half22float2(h);
-                sm += hf.x; sm += hf.y;
-                o4[j] = *reinterpret_cast<const unsigned*>(&h);
-            }
-            og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            ss += __shfl_xor_sync(0xffffffffu, ss, o);
-            sm += __shfl_xor_sync(0xffffffffu, sm, o);
-        }
-        if (lane == 0) { A.xscale[t] = sc_dn; A.xnorm[t] = sqrtf(ss) * sc_dn; A.xsum[t] = sm; }
-    }
-    // scores: warp w takes experts w, w + nwarps, ...; one pass over the expert's row serves all tokens
-    for (int e = warp; e < E; e += nwarps) {
-        float acc[kSingleCtaMaxTokens];
-#pragma unroll
-        for (int t = 0; t < kSingleCtaMaxTokens; ++t) acc[t] = 0.f;
-        for (int i0 = 0; i0 < c8; i0 += 32 * kWB) {
-            if (e != warp || i0 != 0) {                      // later batches: load now (the first one is in registers)
+    for (int le = first; scores && le < n_own; le += slots) {
+        const int e = q + kClusterCtas * le;
+        const float bv = A.bias ? A.bias[e] : 0.f;
+#pragma unroll 1
+        for (int t = tq; t < T; t += g) {
+            float acc = 0.f;
+#pragma unroll 1
+            for (int i0 = 0; i0 < c8; i0 += 32 * kWB) {
+                if (i0 != 0 || (c8 > 32 * kWB ? t != tq || le != first : t == tq && le != first)) fetch(le, i0);
 #pragma unroll
                 for (int j = 0; j < kWB; ++j) {
+                    if (i0 + 32 * j >= c8) break;
                     const int i = i0 + lane + 32 * j;
-                    wpre[j] = (i < c8) ? __ldg(wg + (size_t)e * c8 + i) : make_uint4(0, 0, 0, 0);
+                    if (i < c8) acc = dot8(wpre[j], xs[t * c8 + i], acc);
                 }
             }
-            for (int t = 0; t < T; ++t) {
-                float a = acc[0];                            // rotate so that acc[t] is addressed statically
 #pragma unroll
-                for (int q = 0; q < kSingleCtaMaxTokens; ++q) if (q == t) a = acc[q];
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) {
+                unsigned at;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(&s_sc[t][e])));
+                asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(at), "f"(acc + bv) : "memory");
+            }
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    if (q != 0) {
+        // ---------------------------------------------------- fp16 copies: token t by CTA 1 + t
+        for (int t = q - 1; t < T; t += kClusterCtas - 1) {
+            const uint4* row = xs + t * c8;
+            float m = 0.f;
+            for (int i = threadIdx.x; i < c8; i += kClusterThreads) {
+                const uint4 v = row[i];
+                const unsigned w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int j = 0; j < kWB; ++j) {
-                    const int i = i0 + lane + 32 * j;
-                    if (i < c8) a = dot8(wpre[j], xs[t * c8 + i], a);
+                for (int j = 0; j < 4; ++j) m = fmaxf(m, fmaxf(fabsf(bf16lo(w4[j])), fabsf(bf16hi(w4[j]))));
+            }
+            m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+            if (lane == 0) s_red[0][warp] = m;
+            __syncthreads();
+            m = s_red[0][lane & (kWarps - 1)];
+            m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+            int ex = expo_of(m);
+            ex = (m > 0.f) ? max(-100, min(127, ex)) : 13;
+            const float sc_up = __uint_as_float((unsigned)(127 + 13 - ex) << 23);   // row maximum -> [2^13, 2^14)
+            const float sc_dn = __uint_as_float((unsigned)(127 - 13 + ex) << 23);
+            float ss = 0.f, sm = 0.f;
+            uint4* og = reinterpret_cast<uint4*>(A.x16) + (size_t)t * c8;
+            for (int i = threadIdx.x; i < c8; i += kClusterThreads) {
+                const uint4 v = row[i];
+                const unsigned w4[4] = {v.x, v.y, v.z, v.w};
+                unsigned o4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float a = bf16lo(w4[j]) * sc_up, b = bf16hi(w4[j]) * sc_up;
+                    ss = fmaf(a, a, ss); ss = fmaf(b, b, ss);
+                    const __half2 h = __floats2half2_rn(a, b);
+                    const float2 hf = __half22float2(h);
+                    sm += hf.x; sm += hf.y;
+                    o4[j] = *reinterpret_cast<const unsigned*>(&h);
                 }
-#pragma unroll
-                for (int q = 0; q < kSingleCtaMaxTokens; ++q) if (q == t) acc[q] = a;
+                og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
             }
-        }
-        const float bv = (e == warp) ? bpre : (A.bias ? A.bias[e] : 0.f);
 #pragma unroll
-        for (int t = 0; t < kSingleCtaMaxTokens; ++t) {
-            if (t < T) {
-#pragma unroll
-                for (int o = 16; o; o >>= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
-                if (lane == 0) s_sc[t][e] = acc[t] + bv;
+            for (int o = 16; o; o >>= 1) {
+                ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                sm += __shfl_xor_sync(0xffffffffu, sm, o);
             }
+            if (lane == 0) { s_red[1][warp] = ss; s_red[2][warp] = sm; }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                float a = 0.f, b = 0.f;
+                for (int i = 0; i < kWarps; ++i) { a += s_red[1][i]; b += s_red[2][i]; }
+                A.xscale[t] = sc_dn; A.xnorm[t] = sqrtf(a) * sc_dn; A.xsum[t] = b;
+            }
+            __syncthreads();
         }
-    }
-    __syncthreads();
-    if (A.scores != nullptr)
-        for (int i = threadIdx.x; i < T * E; i += kSingleCtaThreads) A.scores[i] = s_sc[i / E][i % E];
-    for (int t = warp; t < T; t += nwarps) {
-        float v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (lane + 32 * i < E) ? s_sc[t][lane + 32 * i] : -INFINITY;
-        int oi; float ov;
-        warp_topk_lanes(v, E, k, lane, oi, ov);
-        const float wj = topk_softmax(ov, k, lane);
-        if (lane < k) {
-            s_idx[t][lane] = oi;
-            A.idx[(size_t)t * k + lane] = oi;
-            A.wts[(size_t)t * k + lane] = wj;
-        }
-    }
-    __syncthreads();
-    // grouping from shared memory (T <= 8: one ballot per expert)
-    for (int e = warp; e < E; e += nwarps) {
-        int jsel = -1;
-        if (lane < T)
-            for (int j = 0; j < k; ++j) if (s_idx[lane][j] == e) { jsel = j; break; }
-        const unsigned m = __ballot_sync(0xffffffffu, jsel >= 0);
-        if (jsel >= 0) s_rank[lane][jsel] = __popc(m & ((1u << lane) - 1u));
-        if (lane == 0) s_count[e] = __popc(m);
-    }
-    for (int s = threadIdx.x; s < ns; s += kSingleCtaThreads) s_count[E + s] = T;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int a = 0;
-        for (int e = 0; e < Etot; ++e) { s_off[e] = a; a += s_count[e]; }
-        s_off[Etot] = a;
-    }
-    __syncthreads();
-    notify_host(G, s_count, Etot);
-    for (int e = threadIdx.x; e <= Etot; e += kSingleCtaThreads) {
-        G.offset[e] = s_off[e];
-        if (e < Etot) G.count[e] = s_count[e];
-    }
-    for (int p = threadIdx.x; p < T * kk; p += kSingleCtaThreads) {
-        const int t = p / kk, j = p % kk;
-        const int pos = (j < k) ? s_off[s_idx[t][j]] + s_rank[t][j] : s_off[E + (j - k)] + t;
-        G.perm[p] = pos;
-        G.row_token[pos] = t; G.hmax[pos] = 0u;
-    }
-    if (!A.do_sched) {
-        if (threadIdx.x < 8) G.done_mask[threadIdx.x] = 0u;
+        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
         return;
     }
-    // schedule over all experts: resident ones run, missing ones are flagged
-    if (threadIdx.x < kMaxExperts) {
-        const int e = threadIdx.x;
-        const bool need = e < Etot && s_count[e] > 0;
-        const bool res = need && s_slot[e] >= 0;
-        const unsigned done = __ballot_sync(0xffffffffu, res), miss = __ballot_sync(0xffffffffu, need && !res);
-        if (lane == 0) {
-            S.done_mask[e >> 5] = done;
-            s_word[e >> 5] = done;
-            if (miss && !S.quiet) { atomicOr(S.miss_mask + (e >> 5), miss); atomicOr(S.status, 1); }
-        }
+    // -------------------------------------------------------- CTA 0: selection, grouping, schedule
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    int oi = 0;
+    float ov = 0.f;
+    if (warp < T) {
+        warp_topk_lanes(s_sc[warp], E, k, lane, oi, ov);
+        if (lane < k) s_idx[warp * k + lane] = oi;
     }
     __syncthreads();
-    write_schedule(S, s_word);
+    const int P = T * k;
+    if (warp < kClusterMaxTokens) {
+        if (warp < T) {
+            const float wj = topk_softmax(ov, k, lane);
+            if (lane < k) {
+                A.idx[(size_t)warp * k + lane] = oi;
+                A.wts[(size_t)warp * k + lane] = wj;
+            }
+        }
+        if (A.scores != nullptr)
+            for (int i = threadIdx.x; i < T * E; i += 32 * kClusterMaxTokens) A.scores[i] = s_sc[i / E][i % E];
+    } else {
+        // At most 64 pairs: a thread per expert and one per position count over all of them, nothing is passed on. (This code runs
+        // once per step and is fetched cold, so what counts is its length: with matches, a scan and a barrier after
+        // each this part took 3.1 us.)
+        const int tid = threadIdx.x - 32 * kClusterMaxTokens, n = kClusterThreads - 32 * kClusterMaxTokens;
+        int count = 0;
+        if (tid <= Etot) {
+            int below = 0;
+#pragma unroll 1
+            for (int p = 0; p < P; ++p) { const int x = s_idx[p]; below += x < tid; count += x == tid; }
+            if (tid >= E) { below += T * (tid - E); count = T; }
+            G.offset[tid] = below;
+            if (tid < Etot) {
+                G.count[tid] = count;
+                if (G.host_count != nullptr) G.host_count[tid] = count;
+            } else count = 0;
+        }
+        if (A.do_sched && tid < kMaxExperts) {       // schedule over all experts: resident ones run, missing ones are flagged
+            const bool res = count > 0 && s_slot[tid] >= 0;
+            const unsigned done = __ballot_sync(0xffffffffu, res), miss = __ballot_sync(0xffffffffu, count > 0 && !res);
+            if (lane == 0) {
+                S.done_mask[tid >> 5] = done;
+                s_word[tid >> 5] = done;
+                if (miss && !S.quiet) { atomicOr(S.miss_mask + (tid >> 5), miss); atomicOr(S.status, 1); }
+            }
+        }
+        if (!A.do_sched && tid < 8) G.done_mask[tid] = 0u;
+        for (int p = n - 1 - tid; p < T * kk; p += n) {
+            const int t = p / kk, j = p - t * kk;
+            int pos = P + T * (j - k) + t;
+            if (j < k) {
+                const int own = t * k + j, e = s_idx[own];
+                pos = 0;
+#pragma unroll 1
+                for (int o = 0; o < P; ++o) { const int x = s_idx[o]; pos += x < e || (x == e && o < own); }
+            }
+            G.perm[p] = pos;
+            G.row_token[pos] = t; G.hmax[pos] = 0u;
+        }
+    }
+    if (G.host_count != nullptr) __threadfence_system();
+    __syncthreads();
+    if (G.host_count != nullptr && threadIdx.x == 0) { __threadfence_system(); *G.host_flag = G.host_seq; }
+    if (A.do_sched) write_schedule(S, s_word);
 }
 
 // S7 pooling of per-token scores that the caller asked for: pooled[e] = mean_t score[t][e]; then the k_pred best.
@@ -1053,8 +1078,7 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
     if (fused_schedule) *fused_schedule = 0;
     GroupArgs G = group_args(ctx, T, k, rv);
     if (T <= (E > 16 ? kFusedRouteMaxTokens : kFusedRouteMaxTokensFewExperts)) {
-        // one CTA for everything only while its T * E dot products stay cheap for a single SM
-        const bool single = T <= kSingleCtaMaxTokens && E <= 16 && (size_t)T * C * 2 <= 96 * 1024;
+        const bool cluster = T <= kClusterMaxTokens;          // (the token rows fit: hidden sizes end at 16384)
         TokenArgs A;
         A.x = (const __nv_bfloat16*)x; A.T = T; A.C = C; A.W = (const __nv_bfloat16*)w; A.bias = b; A.E = E;
         A.scores = rv.logits; A.x16 = x16; A.xscale = xscale; A.xnorm = xnorm; A.xsum = ws_ptr<float>(ctx, ctx->lay.xsum);
@@ -1063,12 +1087,15 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
         A.do_sched = slot_map != nullptr;
         A.xq = T > kDirectMax && T <= kTokenOrderMax ? ws_ptr<int8_t>(ctx, ctx->lay.xq) : nullptr;
         A.xq_plane = (size_t)Pmax(ctx->cfg) * C;
-        SchedArgs S = sched_args(ctx, slots, slot_map, nullptr, T, k, single ? 1 : T, quiet_schedule);
+        SchedArgs S = sched_args(ctx, slots, slot_map, nullptr, T, k, cluster ? kClusterCtas : T, quiet_schedule);
         S.n_stat = n_stat;
         S.n_pre = n_stat != 0 && ctx->cfg.n_shared > 0 ? std::max(0, ctx->n_sm - n_stat - S.n_main) : 0;      // the SMs that have no other CTA
         const int extra = S.n_stat + S.n_pre;
         ProfScope ps(ctx, MIRA_K_ROUTE, st);
-        if (single) MIRA_CUDA_OK(launch_pdl(k_route_small, dim3(1 + extra), dim3(kSingleCtaThreads), (size_t)T * C * 2, st, A, G, S));
+        if (cluster) {
+            const int grid = (kClusterCtas + extra + kClusterCtas - 1) / kClusterCtas * kClusterCtas;       // whole clusters; CTAs beyond have nothing to do
+            MIRA_CUDA_OK(launch_pdl(k_route_cluster, dim3(grid), dim3(kClusterThreads), (size_t)T * C * 2, st, A, G, S));
+        }
         else if (E > 16) {                   // a warp per expert and round
             if (T * k <= 64) MIRA_CUDA_OK(launch_pdl(k_route_token<true, 1024>, dim3(T + extra), dim3(1024), token_smem(C, 32, E), st, A, G, S));
             else MIRA_CUDA_OK(launch_pdl(k_route_token<false, 1024>, dim3(T + extra), dim3(1024), token_smem(C, 32, E), st, A, G, S));
@@ -1131,7 +1158,7 @@ mira_status set_route_attributes() {
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<false, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterMaxTokens * 16384 * 2));
     return MIRA_OK;
 }
 
