@@ -712,12 +712,14 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
 // Every score is one warp's sum in the order that the other routing kernels use, so all give the same bits.
 // What bounds it: round trips, and code that is run once per step and fetched cold (from L2 at best): the loops stay rolled and
 // the tail has as few instructions and barriers as it can. Measured, us per step, before (up to 16 experts in one CTA, else a CTA
-// per token and a ticket) -> now: 8x7B shape, 1 token 71.2 -> 69.9, 4: 133.9 -> 130.6; fine-grained layer, 1 token 34.8 -> 30.1, 4: 39.3
-// -> 35.9; 1024 x 512, 16 experts, 4 tokens 24.2 -> 20.0; 200 experts, 2 tokens 40.7 -> 29.8. From the previous step's end on, 8x7B /
+// per token and a ticket) -> now: 8x7B shape, 1 token 71.2 -> 69.9, 4: 133.9 -> 130.6, 8: 191 -> 189; fine-grained layer, 1 token 34.8 -> 30.1, 4: 39.3
+// -> 35.9, 8: 44.8 -> 43.7; 1024 x 512, 16 experts, 4 tokens 24.2 -> 20.0; 200 experts, 2 tokens 40.7 -> 29.8. From the previous step's end on, 8x7B /
 // fine-grained with 4 tokens: rows staged 1.4 / 1.0, scores 3.2 / 3.8, cluster barrier 3.7 / 4.5, selection 4.0 / 5.3, all written 5.3 / 6.8
 // us. Tried: the scores' loops unrolled over the tokens (decode of 8x7B 72.2); warps that run the tail's code once ahead of time
 // (39.2 against 37.2 then: they fetch the same lines from the same place).
-constexpr int kClusterCtas = 8, kClusterThreads = 512, kClusterMaxTokens = 4;
+constexpr int kClusterCtas = 8, kClusterThreads = 512, kClusterMaxTokens = 8;
+static_assert(kClusterThreads - 32 * kClusterMaxTokens >= kMaxExperts, "a thread per expert beside the selecting warps");
+constexpr size_t kClusterSmem = 128 * 1024;           // rows of the batch, at most
 
 __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads) k_route_cluster(const __grid_constant__ TokenArgs A, const __grid_constant__ GroupArgs G, const __grid_constant__ SchedArgs S) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -792,7 +794,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
     if (q != 0) {
-        // ---------------------------------------------------- fp16 copies: token t by CTA 1 + t
+        // ---------------------------------------------------- fp16 copies: token t by CTA 1 + t mod 7 (with digit planes when the up/gate kernel wants them)
         for (int t = q - 1; t < T; t += kClusterCtas - 1) {
             const uint4* row = xs + t * c8;
             float m = 0.f;
@@ -827,6 +829,13 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
                     o4[j] = *reinterpret_cast<const unsigned*>(&h);
                 }
                 og[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+                if (A.xq != nullptr) {
+                    float h[8];
+                    halves8(make_uint4(o4[0], o4[1], o4[2], o4[3]), h);
+                    const Digits8 d = digits8(h, kXDigits);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A.xq + p * A.xq_plane + (size_t)t * C + 8 * i) = d.p[p];
+                }
             }
 #pragma unroll
             for (int o = 16; o; o >>= 1) {
@@ -866,21 +875,22 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
         if (A.scores != nullptr)
             for (int i = threadIdx.x; i < T * E; i += 32 * kClusterMaxTokens) A.scores[i] = s_sc[i / E][i % E];
     } else {
-        // At most 64 pairs: a thread per expert and one per position count over all of them, nothing is passed on. (This code runs
+        // At most 128 pairs: a thread per expert and one per position count over all of them, nothing is passed on. (This code runs
         // once per step and is fetched cold, so what counts is its length: with matches, a scan and a barrier after
         // each this part took 3.1 us.)
         const int tid = threadIdx.x - 32 * kClusterMaxTokens, n = kClusterThreads - 32 * kClusterMaxTokens;
         int count = 0;
-        if (tid <= Etot) {
-            int below = 0;
+        for (int e = tid; e <= Etot; e += n) {
+            int below = 0, c = 0;
 #pragma unroll 1
-            for (int p = 0; p < P; ++p) { const int x = s_idx[p]; below += x < tid; count += x == tid; }
-            if (tid >= E) { below += T * (tid - E); count = T; }
-            G.offset[tid] = below;
-            if (tid < Etot) {
-                G.count[tid] = count;
-                if (G.host_count != nullptr) G.host_count[tid] = count;
-            } else count = 0;
+            for (int p = 0; p < P; ++p) { const int x = s_idx[p]; below += x < e; c += x == e; }
+            if (e >= E) { below += T * (e - E); c = e < Etot ? T : 0; }
+            G.offset[e] = below;
+            if (e < Etot) {
+                G.count[e] = c;
+                if (G.host_count != nullptr) G.host_count[e] = c;
+            }
+            if (e == tid) count = c;
         }
         if (A.do_sched && tid < kMaxExperts) {       // schedule over all experts: resident ones run, missing ones are flagged
             const bool res = count > 0 && s_slot[tid] >= 0;
@@ -1078,7 +1088,7 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
     if (fused_schedule) *fused_schedule = 0;
     GroupArgs G = group_args(ctx, T, k, rv);
     if (T <= (E > 16 ? kFusedRouteMaxTokens : kFusedRouteMaxTokensFewExperts)) {
-        const bool cluster = T <= kClusterMaxTokens;          // (the token rows fit: hidden sizes end at 16384)
+        const bool cluster = T <= kClusterMaxTokens && (size_t)T * C * 2 <= kClusterSmem;
         TokenArgs A;
         A.x = (const __nv_bfloat16*)x; A.T = T; A.C = C; A.W = (const __nv_bfloat16*)w; A.bias = b; A.E = E;
         A.scores = rv.logits; A.x16 = x16; A.xscale = xscale; A.xnorm = xnorm; A.xsum = ws_ptr<float>(ctx, ctx->lay.xsum);
@@ -1158,7 +1168,7 @@ mira_status set_route_attributes() {
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<false, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_token<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterMaxTokens * 16384 * 2));
+    MIRA_CUDA_OK(cudaFuncSetAttribute(k_route_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem));
     return MIRA_OK;
 }
 
