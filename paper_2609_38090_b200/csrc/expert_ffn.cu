@@ -130,21 +130,9 @@ __device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n"
                  ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
-// The weights' loads: first to leave L2. They pass through once (several token tiles re-read them at once), and what they would push
-// out is what every step needs again: the kernels' code, the router, the activations. us per step without and with: 8x7B shape,
-// 1 token 73.4 / 71.1, 4: 138 / 130; fine-grained layer, 4 tokens 41.9 / 39.5, 16: 54.6 / 51.7, 64: 81.3 / 78.8.
-__device__ __forceinline__ uint64_t policy_evict_first() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ void tma_weights_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar, uint64_t policy) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;\n"
-                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
-}
-__device__ __forceinline__ void tma_weights_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar, uint64_t policy) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n"
-                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy) : "memory");
+__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
 }
 // fp32 -> fp16, round to nearest even, values beyond the fp16 range go to +-65504 instead of infinity
 __device__ __forceinline__ unsigned short f32_to_f16_sat(float v) {
@@ -324,7 +312,6 @@ __global__ void __launch_bounds__(threads_of(DIRECT), 1) k_ffn(FfnArgs A, const 
         if (warp == 1 && !after_routing) { pdl_wait(); pdl_launch(); }
         int slot = 0, item = blockIdx.x, drawn = 0;
         const CUtensorMap* last_map = nullptr;
-        const uint64_t policy = policy_evict_first();
         uint32_t ph = 1;
         bool ok = true;
         while (ok) {
@@ -367,8 +354,8 @@ __global__ void __launch_bounds__(threads_of(DIRECT), 1) k_ffn(FfnArgs A, const 
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(nb * box_bytes) : "memory");
                         for (int j = 0; j < nb; ++j) {
                             if (warp == 1) tma_3d(dst + j * box_step, map, (b + j) * kKBox, row, 0, bar);
-                            else if (DOWN) tma_weights_2d(dst + j * box_step, map, (b + j) * kKBox, row, bar, policy);
-                            else tma_weights_3d(dst + j * box_step, map, (b + j) * kKBox, 0, row, bar, policy);
+                            else if (DOWN) tma_2d(dst + j * box_step, map, (b + j) * kKBox, row, bar);
+                            else tma_3d(dst + j * box_step, map, (b + j) * kKBox, 0, row, bar);
                         }
                     }
                     __syncwarp();
