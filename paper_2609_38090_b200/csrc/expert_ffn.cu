@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(threads_of(DIRECT), 1) k_ffn(FfnArgs A, const 
     // kernel in front of this one started, unless they are the kernel in front.
     const bool after_routing = !DOWN && (DIRECT || token_order);
     // In the smallest batches, behind the routing kernel, the table is built twice: first on whatever the last step left, under the wait, so that its code has been
-    // fetched when the numbers arrive (fine-grained layer, 4 tokens 36.0 -> 35.3 us, 8x7B shape, 1 token 70.0 both). Any numbers will
+    // fetched when the numbers arrive (fine-grained layer, 4 tokens 2 % of the step, 8x7B shape, 1 token nothing). Any numbers will
     // do: they index nothing (and the loads pass L1 by, which may not keep the old ones).
     constexpr bool kTwice = DIRECT && !DOWN;
     auto load = [](const auto* p) { return kTwice ? __ldcg(p) : *p; };

@@ -710,13 +710,13 @@ __global__ void __launch_bounds__(THREADS) k_route_token(TokenArgs A, GroupArgs 
 // scores the experts q, q + 8, ... for all tokens; the scores meet in CTA 0 through distributed shared memory (one cluster barrier;
 // no ticket, no fences), which selects, groups and writes the schedule while the others write the fp16 copies of the tokens.
 // Every score is one warp's sum in the order that the other routing kernels use, so all give the same bits.
-// What bounds it: round trips, and code that is run once per step and fetched cold (from L2 at best): the loops stay rolled and
-// the tail has as few instructions and barriers as it can. Measured, us per step, before (up to 16 experts in one CTA, else a CTA
-// per token and a ticket) -> now: 8x7B shape, 1 token 71.2 -> 69.9, 4: 133.9 -> 130.6, 8: 191 -> 189; fine-grained layer, 1 token 34.8 -> 30.1, 4: 39.3
-// -> 35.9, 8: 44.8 -> 43.7; 1024 x 512, 16 experts, 4 tokens 24.2 -> 20.0; 200 experts, 2 tokens 40.7 -> 29.8. From the previous step's end on, 8x7B /
-// fine-grained with 4 tokens: rows staged 1.4 / 1.0, scores 3.2 / 3.8, cluster barrier 3.7 / 4.5, selection 4.0 / 5.3, all written 5.3 / 6.8
-// us. Tried: the scores' loops unrolled over the tokens (decode of 8x7B 72.2); warps that run the tail's code once ahead of time
-// (39.2 against 37.2 then: they fetch the same lines from the same place).
+// What bounds it: round trips, and code that is run once per step and fetched cold: the loops stay rolled and the tail has as few
+// instructions and barriers as it can. Measured, us per step, before (one CTA for up to 4 tokens and 16 experts, else a CTA
+// per token and a ticket) -> now: 8x7B shape, 1 token 73.4 -> 71.9, 4: 137 -> 133, 8: 195 -> 193; fine-grained layer (60 experts), 1
+// token 35.8 -> 29.6, 4: 41.9 -> 37.0; 1024 x 512, 16 experts, 4 tokens 24.3 -> 19.2; 200 experts, 2 tokens 41.2 -> 28.9. More experts
+// with more tokens are too many scores for eight SMs: fine-grained layer, 8 tokens 47.2 a CTA per token, 47.6 here. Tried: the
+// scores' loops unrolled over the tokens (8x7B shape, 1 token 76); warps that run the tail's code once ahead of time (slower by
+// 2 us: they fetch the same lines from the same place).
 constexpr int kClusterCtas = 8, kClusterThreads = 512, kClusterMaxTokens = 8;
 static_assert(kClusterThreads - 32 * kClusterMaxTokens >= kMaxExperts, "a thread per expert beside the selecting warps");
 constexpr size_t kClusterSmem = 128 * 1024;           // rows of the batch, at most
@@ -877,7 +877,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     } else {
         // At most 128 pairs: a thread per expert and one per position count over all of them, nothing is passed on. (This code runs
         // once per step and is fetched cold, so what counts is its length: with matches, a scan and a barrier after
-        // each this part took 3.1 us.)
+        // each this part took 3.1 us, now 0.8.)
         const int tid = threadIdx.x - 32 * kClusterMaxTokens, n = kClusterThreads - 32 * kClusterMaxTokens;
         int count = 0;
         for (int e = tid; e <= Etot; e += n) {
@@ -1088,7 +1088,7 @@ mira_status launch_route(mira_ctx* ctx, const void* x, int T, const void* w, con
     if (fused_schedule) *fused_schedule = 0;
     GroupArgs G = group_args(ctx, T, k, rv);
     if (T <= (E > 16 ? kFusedRouteMaxTokens : kFusedRouteMaxTokensFewExperts)) {
-        const bool cluster = T <= kClusterMaxTokens && (size_t)T * C * 2 <= kClusterSmem;
+        const bool cluster = T <= (E <= 16 ? kClusterMaxTokens : 4) && (size_t)T * C * 2 <= kClusterSmem;      // (see k_route_cluster)
         TokenArgs A;
         A.x = (const __nv_bfloat16*)x; A.T = T; A.C = C; A.W = (const __nv_bfloat16*)w; A.bias = b; A.E = E;
         A.scores = rv.logits; A.x16 = x16; A.xscale = xscale; A.xnorm = xnorm; A.xsum = ws_ptr<float>(ctx, ctx->lay.xsum);

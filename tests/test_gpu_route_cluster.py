@@ -1,4 +1,4 @@
-"""Routing of 1 to 8 tokens by one cluster of CTAs: numbers of experts around multiples of the cluster's size and of a warp's lanes,
+"""Routing of 1 to 4 tokens, and of up to 8 with at most 16 experts, by one cluster of CTAs: numbers of experts around multiples of the cluster's size and of a warp's lanes,
 hidden sizes around a warp's registers (512 vectors of eight), small and large top-k, shared experts; against the oracle, and the same scores
 bit for bit as in a batch that another kernel routes."""
 import numpy as np
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("T,C,E,k,ns", [(1, 64, 1, 1, 0), (4, 64, 7, 7, 1), (3, 192, 8, 2, 0), (2, 512, 9, 3, 3), (4, 2048, 60, 4, 4), (1, 4096, 8, 2, 0),
                                         (4, 4160, 17, 16, 0), (2, 8192, 33, 5, 2), (3, 16384, 65, 6, 0), (4, 1024, 127, 16, 1), (4, 320, 240, 8, 16),
-                                        (5, 2048, 60, 4, 4), (8, 192, 240, 16, 16), (7, 8192, 16, 2, 0), (8, 8192, 9, 9, 1), (8, 4096, 8, 2, 0)])
+                                        (4, 192, 240, 16, 16), (5, 2048, 16, 4, 4), (7, 8192, 16, 2, 0), (8, 8192, 9, 9, 1), (8, 4096, 8, 2, 0)])
 def test_route_cluster(T, C, E, k, ns):
     from paper_2609_38090_b200 import binding as b
     g = np.random.default_rng(C + E)
