@@ -34,7 +34,7 @@
 // themselves (cp.async, 16 bytes a request) leaving out their copies and conversion took a quarter of its time away, the
 // conversion alone 2 to 4 %. TMA boxes move the same bytes for less energy and off the converters' chain. us per step, before
 // -> now: 8x7B 1200 tokens 1095 -> 1030, 2048: 1701 -> 1570, 3072: 2530 -> 2330; fine-grained layer 1000 tokens 328 -> 306, 256
-// tokens 144 -> 146. Left out on trial (2048 / 1000 tokens, 1625 / 318 us in that run): conversion 1556 / 307, the weights'
+// tokens 144 -> 143.5. Left out on trial (2048 / 1000 tokens, 1625 / 318 us in that run): conversion 1556 / 307, the weights'
 // boxes too 1373 / 281, the activations' boxes 1436 / 295, tcgen05.st nothing: what moves from L2 counts most.
 // Tried and dropped: one lane that serves both rings, blocking on each in turn (3 to 10 % slower) or polling them (4 %); two
 // pairs of SMs' clusters per SM pair, so that each SM loads half of the activations (no gain: the higher clock pays for the
@@ -367,10 +367,12 @@ __global__ void __launch_bounds__(TC::kThreads, TC::kCtasPerSm) k_ffn_tc(TcArgs 
     const uint32_t tmem = s_tmem;
     const long total = (long)s_ntile[s_nact] * per_e;     // < 2^31
     // Everything above read only what the routing kernels wrote, and those had completed before the kernel in front
-    // of this one started (it waited for them before letting this one launch). The activations come from that
-    // kernel itself.
-    pdl_wait();
-    pdl_launch();
+    // of this one started (it waited for them before letting this one launch). The same holds for the weights and their maps, so the
+    // weight warp and the converters begin at once; the activations come from the kernel in front itself, and what the epilogue
+    // overwrites it may still read. (Step of the fine-grained layer, 256 tokens 145.9 -> 143.5 us, 8x7B shape, 600 tokens 689 -> 686; 1000
+    // and 2048 tokens the same.)
+    if (warp >= kEpiWarp0 && warp <= kTmaWarp) pdl_wait();
+    if (warp == kTmaWarp) pdl_launch();
 
     // tile order: (expert, slice, row block, token tile) with the token tile fastest, so CTAs working at the same
     // time share weight rows through L2
